@@ -2151,14 +2151,76 @@ __device__ __forceinline__ void merge_batch(const MergeArgs& a, int qh, int lane
             if (srcs[u]) l2_discard(srcs[u]);
 }
 
+// Fold cnt (1..32) partial rows into the running (M, L, acc) of a row: lane k
+// holds slot k (lanes past cnt: any valid slot) and whether its index is
+// good. The LSEs and the first four rows are loaded together.
 template <int HD>
-__global__ void __launch_bounds__(128) merge_kernel(const MergeArgs a) {
+__device__ __forceinline__ void merge_chunk(const MergeArgs& a, int qh, int lane, int slot, bool ok, int cnt,
+                                            uint64_t pol, float& M, float& L, float (&acc)[HD / 32]) {
+    constexpr int DPL = HD / 32;
+    float x0[4][DPL];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int64_t sl = __shfl_sync(0xffffffffu, slot, u < cnt ? u : 0);
+        const float* src = a.part_o + (sl * a.hq + qh) * HD + lane * DPL;
+        if constexpr (DPL == 4) {
+            const float4 v = ld_f4_hint(src, pol);
+            x0[u][0] = v.x, x0[u][1] = v.y, x0[u][2] = v.z, x0[u][3] = v.w;
+        } else {
+            const float2 v = ld_f2_hint(src, pol);
+            x0[u][0] = v.x, x0[u][1] = v.y;
+        }
+    }
+    const float lse = lane < cnt && ok ? a.part_lse[(int64_t)slot * a.hq + qh] : -INFINITY;
+    float cm = lse;
+#pragma unroll
+    for (int off = 16; off; off >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, off));
+    const float m_new = fmaxf(M, cm);
+    const float keep = (M == -INFINITY) ? 0.f : fast_exp2(M - m_new);
+    M = m_new;
+    const float w = lane < cnt ? fast_exp2(lse - M) : 0.f;
+    float ws = w;
+#pragma unroll
+    for (int off = 16; off; off >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, off);
+    L = L * keep + ws;
+#pragma unroll
+    for (int d = 0; d < DPL; ++d) acc[d] *= keep;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const float wu = __shfl_sync(0xffffffffu, w, u) * (u < cnt ? 1.f : 0.f);
+#pragma unroll
+        for (int d = 0; d < DPL; ++d) acc[d] += wu * x0[u][d];
+    }
+    constexpr int kLanesPerLine = 128 / (DPL * 4);
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int64_t sl = __shfl_sync(0xffffffffu, slot, u < cnt ? u : 0);  // every lane shuffles
+        if (u < cnt && (lane & (kLanesPerLine - 1)) == 0) l2_discard(a.part_o + (sl * a.hq + qh) * HD + lane * DPL);
+    }
+    for (int j = 4; j < cnt; j += 4) merge_batch<HD>(a, qh, lane, slot, w, j, cnt, pol, acc);
+}
+
+// One row = one (occurrence, q-head). WPR warps share a row: each folds its
+// share of the row's partials, then (WPR > 1) the shares meet in shared
+// memory. What bounds a row is its chain of dependent round trips (slot list,
+// then LSEs and four partial rows at a time), so a call of few rows with many
+// partials each (a few long paths) spreads every row over up to 8 warps;
+// calls whose rows fill the GPU keep one warp per row (see launch_merge).
+// Whole calls, one warp per row against shared rows: one 60k-token path (28
+// rows of 210 partials) 64.2 -> 37.5 us, one 8k path (27 partials) 19.0 ->
+// 16.6, four 8k paths 38.1 -> 34.8; 1024 paths (7 partials, one warp) equal.
+template <int HD, int WPR>
+__global__ void __launch_bounds__(WPR > 4 ? WPR * 32 : 128) merge_kernel(const MergeArgs a) {
     constexpr int DPL = HD / 32;  // dims per lane: 4 or 2
-    const int warp_global = blockIdx.x * 4 + (threadIdx.x >> 5);
+    constexpr int kWarps = WPR > 4 ? WPR : 4;
+    const int warp = threadIdx.x >> 5, part = warp % WPR;
+    const int64_t row = (int64_t)blockIdx.x * (kWarps / WPR) + warp / WPR;
     const int lane = threadIdx.x & 31;
     if (blockIdx.x == 0 && threadIdx.x < 3) a.counters[threadIdx.x] = 0;  // decode is done: re-arm its counters
-    if (warp_global >= a.n * a.hq) return;
-    const int i = warp_global / a.hq, qh = warp_global % a.hq;
+    const bool in_grid = row < (int64_t)a.n * a.hq;
+    if (WPR == 1 && !in_grid) return;
+    const int i = in_grid ? (int)(row / a.hq) : 0, qh = (int)(row % a.hq);
     float acc[DPL];
 #pragma unroll
     for (int d = 0; d < DPL; ++d) acc[d] = 0.f;
@@ -2166,92 +2228,61 @@ __global__ void __launch_bounds__(128) merge_kernel(const MergeArgs a) {
     const uint64_t pol = l2_evict_first();  // each partial row is read once
     // The occurrence's merge record, in one round trip: lane k < 16 holds
     // word k ([count, slots...]).
-    const int rw = a.merge_rec && lane < kMergeRecWords ? a.merge_rec[(int64_t)i * kMergeRecWords + lane] : -1;
+    const int rw =
+        in_grid && a.merge_rec && lane < kMergeRecWords ? a.merge_rec[(int64_t)i * kMergeRecWords + lane] : -1;
     const int ns_rec = __shfl_sync(0xffffffffu, rw, 0);  // -1: the CSR (more than 15 slots, or no records)
+    int ns = 0;
     if (ns_rec >= 0) {
-        // up to 15 slots: lane k takes slot k; its LSE and the first four
-        // partial rows are loaded together, then folded
-        const int ns = ns_rec;
-        if (!check(ns < kMergeRecWords, a.err) || ns == 0) return;  // 0: written directly by its only unit
-        int slot = __shfl_sync(0xffffffffu, rw, (lane + 1) & 31);  // every lane shuffles
-        const int first = __shfl_sync(0xffffffffu, rw, 1);
-        if (lane >= ns)
+        // up to 15 slots: lane k takes slot k of this warp's share
+        ns = check(ns_rec < kMergeRecWords, a.err) ? ns_rec : 0;
+        const int k0 = ns * part / WPR, cnt = ns * (part + 1) / WPR - k0;
+        int slot = __shfl_sync(0xffffffffu, rw, (k0 + lane + 1) & 31);  // every lane shuffles
+        const int first = __shfl_sync(0xffffffffu, slot, 0);
+        if (lane >= cnt)
             slot = first;  // a valid row (weight 0)
         else if (!check(in_range(slot, a.n_slots), a.err))
             slot = 0;
-        float x0[4][DPL];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int64_t sl = __shfl_sync(0xffffffffu, slot, u < ns ? u : 0);
-            const float* src = a.part_o + (sl * a.hq + qh) * HD + lane * DPL;
-            if constexpr (DPL == 4) {
-                const float4 v = ld_f4_hint(src, pol);
-                x0[u][0] = v.x, x0[u][1] = v.y, x0[u][2] = v.z, x0[u][3] = v.w;
-            } else {
-                const float2 v = ld_f2_hint(src, pol);
-                x0[u][0] = v.x, x0[u][1] = v.y;
-            }
-        }
-        const float lse = lane < ns ? a.part_lse[(int64_t)slot * a.hq + qh] : -INFINITY;
-        M = lse;
-#pragma unroll
-        for (int off = 16; off; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
-        const float w = lane < ns ? fast_exp2(lse - M) : 0.f;
-        L = w;
-#pragma unroll
-        for (int off = 16; off; off >>= 1) L += __shfl_xor_sync(0xffffffffu, L, off);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float wu = __shfl_sync(0xffffffffu, w, u) * (u < ns ? 1.f : 0.f);
-#pragma unroll
-            for (int d = 0; d < DPL; ++d) acc[d] += wu * x0[u][d];
-        }
-        {
-            constexpr int kLanesPerLine = 128 / (DPL * 4);
-            __syncwarp();
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t sl = __shfl_sync(0xffffffffu, slot, u < ns ? u : 0);  // every lane shuffles
-                if (u < ns && (lane & (kLanesPerLine - 1)) == 0) l2_discard(a.part_o + (sl * a.hq + qh) * HD + lane * DPL);
-            }
-        }
-        for (int j = 4; j < ns; j += 4) merge_batch<HD>(a, qh, lane, slot, w, j, ns, pol, acc);
-    } else {
-        // more slots: the CSR, in chunks of 32 -- lane k fetches slot k's
-        // index and LSE, then the warp folds the chunk's partial rows, four
-        // loads in flight per lane
-        const int beg = a.merge_off[i], ns = a.merge_off[i + 1] - beg;
-        if (!check(merge_range_ok(beg, beg + ns, a.n_merge) && (ns == 0 || a.n_slots > 0), a.err)) return;
-        if (ns == 0) return;
-        for (int c0 = 0; c0 < ns; c0 += 32) {
-            const int k = c0 + lane;
-            int slot = 0;
-            float lse = -INFINITY;
-            if (k < ns) {
-                slot = a.merge_slot[beg + k];
-                if (check(in_range(slot, a.n_slots), a.err))
-                    lse = a.part_lse[(int64_t)slot * a.hq + qh];
-                else
-                    slot = 0;  // weight 0, a valid row to read
-            }
-            float cm = lse;
-#pragma unroll
-            for (int off = 16; off; off >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, off));
-            const float m_new = fmaxf(M, cm);
-            const float keep = (M == -INFINITY) ? 0.f : fast_exp2(M - m_new);
-#pragma unroll
-            for (int d = 0; d < DPL; ++d) acc[d] *= keep;
-            L *= keep;
-            M = m_new;
-            const float w = (k < ns) ? fast_exp2(lse - M) : 0.f;
-            float ws = w;
-#pragma unroll
-            for (int off = 16; off; off >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, off);
-            L += ws;
-            const int cnt = min(32, ns - c0);
-            for (int j = 0; j < cnt; j += 4) merge_batch<HD>(a, qh, lane, slot, w, j, cnt, pol, acc);
+        if (cnt > 0) merge_chunk<HD>(a, qh, lane, slot, true, cnt, pol, M, L, acc);
+    } else if (in_grid) {
+        // more slots: the CSR, in chunks of 32 slots of this warp's share
+        const int beg = a.merge_off[i], all = a.merge_off[i + 1] - beg;
+        ns = check(merge_range_ok(beg, beg + all, a.n_merge) && (all == 0 || a.n_slots > 0), a.err) ? all : 0;
+        const int k0 = (int)((int64_t)ns * part / WPR), k1 = (int)((int64_t)ns * (part + 1) / WPR);
+        for (int c0 = k0; c0 < k1; c0 += 32) {
+            const int cnt = min(32, k1 - c0);
+            int slot = a.merge_slot[beg + c0 + min(lane, cnt - 1)];
+            const bool ok = check(in_range(slot, a.n_slots), a.err);
+            if (!ok) slot = 0;  // weight 0, a valid row to read
+            merge_chunk<HD>(a, qh, lane, slot, ok, cnt, pol, M, L, acc);
         }
     }
+    if constexpr (WPR > 1) {
+        __shared__ float s_acc[kWarps][HD];
+        __shared__ float s_m[kWarps], s_l[kWarps];
+        if (part != 0) {
+#pragma unroll
+            for (int d = 0; d < DPL; ++d) s_acc[warp][lane * DPL + d] = acc[d];
+            if (lane == 0) s_m[warp] = M, s_l[warp] = L;
+        }
+        __syncthreads();
+        if (part != 0 || !in_grid) return;
+        float Mw = M;
+#pragma unroll
+        for (int k = 1; k < WPR; ++k) Mw = fmaxf(Mw, s_m[warp + k]);
+        const float w0 = M == -INFINITY ? 0.f : fast_exp2(M - Mw);
+#pragma unroll
+        for (int d = 0; d < DPL; ++d) acc[d] *= w0;
+        L *= w0;
+#pragma unroll
+        for (int k = 1; k < WPR; ++k) {
+            const float wk = s_m[warp + k] == -INFINITY ? 0.f : fast_exp2(s_m[warp + k] - Mw);
+            L += wk * s_l[warp + k];
+#pragma unroll
+            for (int d = 0; d < DPL; ++d) acc[d] += wk * s_acc[warp + k][lane * DPL + d];
+        }
+        M = Mw;
+    }
+    if (ns == 0) return;  // written directly by its only unit
     const float inv = 1.f / L;
     uint16_t* dst = a.out + ((int64_t)i * a.hq + qh) * HD + lane * DPL;
     if constexpr (DPL == 4) {
@@ -2492,14 +2523,34 @@ cudaError_t launch_decode(int hd, const DecodeArgs& a, cudaStream_t s, cudaStrea
     return hd == 64 ? launch_decode_hd<64>(a, s, side, fork, join) : launch_decode_hd<128>(a, s, side, fork, join);
 }
 
-cudaError_t launch_merge(int hd, const MergeArgs& a, cudaStream_t s) {
-    const int64_t warps = (int64_t)a.n * a.hq;
-    const int grid = (int)std::max<int64_t>(1, (warps + 3) / 4);  // one block at least: it re-arms the counters
+namespace {
+template <int WPR>
+cudaError_t launch_merge_wpr(int hd, const MergeArgs& a, cudaStream_t s) {
+    constexpr int kWarps = WPR > 4 ? WPR : 4;
+    const int64_t warps = (int64_t)a.n * a.hq * WPR;
+    const int grid = (int)std::max<int64_t>(1, (warps + kWarps - 1) / kWarps);  // one block at least: it re-arms the counters
     if (hd == 64)
-        merge_kernel<64><<<grid, 128, 0, s>>>(a);
+        merge_kernel<64, WPR><<<grid, kWarps * 32, 0, s>>>(a);
     else
-        merge_kernel<128><<<grid, 128, 0, s>>>(a);
+        merge_kernel<128, WPR><<<grid, kWarps * 32, 0, s>>>(a);
     return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_merge(int hd, const MergeArgs& a, cudaStream_t s) {
+    // Warps per row: the fewest (1, 2, 4, 8) that leave a warp at most four
+    // partials on average (one batch of loads in flight), as long as all warps
+    // are resident at once (about 32 per SM): past that, more warps only queue.
+    const int64_t rows = (int64_t)a.n * a.hq;
+    const int64_t avg = a.n > 0 ? (a.n_merge + a.n - 1) / a.n : 0;  // partials of a row
+    int wpr = 1;
+    while (wpr < 8 && avg > 4 * wpr && rows * wpr * 2 <= 152 * 32) wpr *= 2;
+    switch (wpr) {
+        case 1: return launch_merge_wpr<1>(hd, a, s);
+        case 2: return launch_merge_wpr<2>(hd, a, s);
+        case 4: return launch_merge_wpr<4>(hd, a, s);
+        default: return launch_merge_wpr<8>(hd, a, s);
+    }
 }
 
 }  // namespace tp
