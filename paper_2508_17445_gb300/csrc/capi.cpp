@@ -894,11 +894,15 @@ tp_status tp_decode_noalloc(tp_tree* t, const tp_node* leaves, int32_t n, const 
     if (cap != cudaStreamCaptureStatusNone)
         return fail(t, TP_ERR_INVALID_ARG, "tp_decode_noalloc cannot run while its stream is being captured");
     tp::Schedule S;  // host-side only; the tree's schedule cache is left alone
-    tp_status st = tp::build_schedule(t, leaves, n, flags & ~TP_DECODE_NO_CACHE, S);
-    if (st != TP_OK) return st;
     const int32_t hq = t->cfg.num_q_heads, hd = t->cfg.head_dim;
-    const int64_t sched_bytes = ((int64_t)S.words.size() * 4 + 255) / 256 * 256;
-    const int64_t part_bytes = (int64_t)S.n_slots * hq * (hd + 1) * 4;
+    int64_t sched_bytes = 0, part_bytes = 0;
+    for (const bool coarse : {false, true}) {  // the schedule with the fewest partials where the other does not fit
+        tp_status st = tp::build_schedule(t, leaves, n, flags & ~TP_DECODE_NO_CACHE, S, coarse);
+        if (st != TP_OK) return st;
+        sched_bytes = ((int64_t)S.words.size() * 4 + 255) / 256 * 256;
+        part_bytes = (int64_t)S.n_slots * hq * (hd + 1) * 4;
+        if (sched_bytes + part_bytes <= TP_NOALLOC_SCRATCH_BYTES) break;
+    }
     if (sched_bytes + part_bytes > TP_NOALLOC_SCRATCH_BYTES)
         return fail(t, TP_ERR_OOM,
                     "tp_decode_noalloc needs " + std::to_string(sched_bytes + part_bytes) +

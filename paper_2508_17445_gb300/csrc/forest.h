@@ -468,7 +468,10 @@ tp_status rollout_token_step(tp_tree* t, const tp_node* nodes, int32_t n, int32_
 // forest.cpp
 tp_status fail(tp_tree* t, tp_status code, const std::string& msg);
 tp_status check_live(tp_tree* t, tp_node node, bool need_leaf);
-tp_status build_schedule(tp_tree* t, const tp_node* leaves, int32_t n, uint32_t flags, Schedule& out);
+// coarse: units as long as the partials' share of the traffic asks for, also
+// where that leaves the GPU partly idle (the fewest partials).
+tp_status build_schedule(tp_tree* t, const tp_node* leaves, int32_t n, uint32_t flags, Schedule& out,
+                         bool coarse = false);
 // Prefill: the last m[i] tokens of nodes[i] attend causally to their root-
 // to-node path. Occurrence q (query token, packed node by node) sees the
 // path's first vis[q] tokens; its rows are kept per node in blocks of whole
