@@ -131,37 +131,51 @@ void append_tokens_commit(tp_tree* t, const tp_node* nodes, int32_t n, int64_t n
     if (need > 0) ++t->struct_version;
 }
 
-// One token step of the rollout's decode loop in one upload and one launch:
-// append a token to each of nodes[0..n) with the stand-in activations of
-// (seed, pos), Q of the rows into q; and, when the cached decode schedule is
-// the one for exactly these nodes and the append stays inside their last
-// blocks, the schedule patch the next tp_decode_ex(decode_flags) would apply.
-// d_buf: device int32 scratch of at least 4 n words.
-tp_status rollout_token_step(tp_tree* t, const tp_node* nodes, int32_t n, int32_t* d_buf, int64_t buf_words,
-                             uint64_t seed, int32_t pos, uint16_t* q, uint32_t decode_flags) {
+int32_t step_patch(tp_tree* t, const tp_node* nodes, int32_t n, bool stays, uint64_t before, bool* patched) {
+    *patched = stays && t->sched_valid && t->sched_version == before && t->sched_struct == t->struct_version &&
+               t->sched_stream == t->stream && t->sched_leaves.size() == (size_t)n && std::equal(nodes, nodes + n, t->sched_leaves.begin());
+    return *patched ? patch_schedule(t, t->sched, t->patch_words) : 0;
+}
+
+tp_status step_words(tp_tree* t, const std::vector<int32_t>& words, StepWords* out) {
+    out->host = words.data();
+    out->n = (int64_t)words.size();
+    if (out->n <= kParamWords) return TP_OK;
+    void* p = t->d_step;
+    int64_t bytes = t->d_step_cap * 4;
+    tp_status st = ensure_device_bytes(t, &p, &bytes, out->n * 4, "token-step words");
+    t->d_step = (int32_t*)p;
+    t->d_step_cap = bytes / 4;
+    if (st == TP_OK) st = stage_upload(t, t->d_step, words.data(), out->n);
+    out->device = t->d_step;
+    return st;
+}
+
+// One token step of the rollout's decode loop in one launch: append a token
+// to each of nodes[0..n) with the stand-in activations of (seed, pos), Q of
+// the rows into q; and the patch of the cached decode schedule that the next
+// tp_decode_ex(decode_flags) would apply (see step_patch).
+tp_status rollout_token_step(tp_tree* t, const tp_node* nodes, int32_t n, uint64_t seed, int32_t pos, uint16_t* q,
+                             uint32_t decode_flags) {
     if (n == 0) return TP_OK;
     int64_t need = 0;
     tp_status st = append_tokens_plan(t, nodes, n, &need);
     if (st != TP_OK) return st;
-    const uint32_t key = decode_flags & ~TP_DECODE_NO_CACHE;
-    const bool patch = !(decode_flags & TP_DECODE_NO_CACHE) && need == 0 && t->sched_valid &&
-                       t->sched_flags == key && t->sched_version == t->version &&
-                       t->sched_struct == t->struct_version && t->sched_leaves.size() == (size_t)n &&
-                       std::equal(nodes, nodes + n, t->sched_leaves.begin()) &&
-                       2 * (int64_t)n + (int64_t)t->sched.leaf_tail.size() <= buf_words;
+    const bool stays = need == 0 && !(decode_flags & TP_DECODE_NO_CACHE) &&
+                       t->sched_flags == (decode_flags & ~TP_DECODE_NO_CACHE);
+    const uint64_t before = t->version;
     append_tokens_commit(t, nodes, n, need);
-    const int32_t n_pairs = patch ? patch_schedule(t, t->sched, t->patch_words) : 0;
+    bool patch = false;
+    const int32_t n_pairs = step_patch(t, nodes, n, stays, before, &patch);
     std::vector<int32_t>& w = t->scratch.step_words;  // row nodes | pool slots | patch pairs
     w.assign(nodes, nodes + n);
     w.insert(w.end(), t->tok_slots.begin(), t->tok_slots.end());
     if (n_pairs > 0) w.insert(w.end(), t->patch_words.begin(), t->patch_words.begin() + 2 * (int64_t)n_pairs);
-    st = (int64_t)w.size() <= buf_words ? stage_upload(t, d_buf, w.data(), (int64_t)w.size())
-                                        : fail(t, TP_ERR_INVALID_ARG, "rollout step buffer too small");
+    StepWords words;
+    st = step_words(t, w, &words);
     if (st == TP_OK) {
         StepArgs a;
-        a.row_node = d_buf;
-        a.slots = d_buf + n;
-        a.pairs = d_buf + 2 * n;
+        a.words = nullptr;
         a.sched = t->d_sched;
         a.pool = (uint8_t*)t->cfg.pool;
         a.q = q;
@@ -177,7 +191,7 @@ tp_status rollout_token_step(tp_tree* t, const tp_node* nodes, int32_t n, int32_
         a.pool_blocks = t->cfg.pool_blocks;
         a.sched_words = (int64_t)t->sched.words.size();
         LaunchTimer timer(t, KK_APPEND);
-        cudaError_t e = launch_rollout_step(t->cfg.head_dim, a, t->stream);
+        cudaError_t e = launch_rollout_step(t->cfg.head_dim, a, words, t->stream);
         if (e != cudaSuccess) st = cuda_fail(t, e, "rollout step kernel");
     }
     if (st != TP_OK) {  // back to the state before the call; the cached schedule is rebuilt next time
@@ -243,11 +257,11 @@ tp_status upload_schedule(tp_tree* t, const tp::Schedule& s) {
 tp_status patch_cached_schedule(tp_tree* t) {
     const int32_t n = tp::patch_schedule(t, t->sched, t->patch_words);
     if (n == 0) return TP_OK;
-    tp_status st = ensure_device(t, t->d_patch, t->d_patch_cap, 2 * (int64_t)n, "schedule patch buffer");
+    t->scratch.step_words.assign(t->patch_words.begin(), t->patch_words.begin() + 2 * (int64_t)n);
+    tp::StepWords words;
+    tp_status st = tp::step_words(t, t->scratch.step_words, &words);
     if (st != TP_OK) return st;
-    st = stage_upload(t, t->d_patch, t->patch_words.data(), 2 * (int64_t)n);
-    if (st != TP_OK) return st;
-    cudaError_t e = tp::launch_patch(t->d_sched, t->d_patch, n, t->stream, (int64_t)t->sched.words.size(), t->d_err);
+    cudaError_t e = tp::launch_patch(t->d_sched, words, n, t->stream, (int64_t)t->sched.words.size(), t->d_err);
     tp::count_kernels(t, tp::KK_DECODE, 1);
     if (e != cudaSuccess) return cuda_fail(t, e, "schedule patch kernel");
     return TP_OK;
@@ -339,8 +353,7 @@ tp_status tp_tree_destroy(tp_tree* t) {
     if (t->d_sched) cudaFree(t->d_sched);
     if (t->d_part) cudaFree(t->d_part);
     if (t->d_gather_tiles) cudaFree(t->d_gather_tiles);
-    if (t->d_patch) cudaFree(t->d_patch);
-    if (t->d_tok_slots) cudaFree(t->d_tok_slots);
+    if (t->d_step) cudaFree(t->d_step);
     for (cudaEvent_t e : t->ev_pool) cudaEventDestroy(e);
     if (t->ev_fork) cudaEventDestroy(t->ev_fork);
     if (t->ev_join) cudaEventDestroy(t->ev_join);
@@ -463,32 +476,46 @@ tp_status tp_append_tokens(tp_tree* t, const tp_node* nodes, int32_t n, const vo
     int64_t need = 0;
     tp_status st = tp::append_tokens_plan(t, nodes, n, &need);
     if (st != TP_OK) return st;
-    if (t->cfg.pool) {
-        const int32_t bt = t->cfg.block_tokens;
-        st = ensure_device(t, t->d_tok_slots, t->d_tok_slots_cap, n, "token slot buffer");
-        if (st == TP_OK) st = stage_upload(t, t->d_tok_slots, t->tok_slots.data(), n);
-        if (st == TP_OK) {
-            tp::AppendTokensArgs a;
-            a.k = K;
-            a.v = V;
-            a.slots = t->d_tok_slots;
-            a.pool = (uint8_t*)t->cfg.pool;
-            a.head_bytes = bt * t->cfg.head_dim * 2;
-            a.block_bytes = (int64_t)2 * t->cfg.num_kv_heads * a.head_bytes;
-            a.hkv = t->cfg.num_kv_heads;
-            a.n = n;
-            a.err = t->d_err;
-            a.pool_blocks = t->cfg.pool_blocks;
-            tp::LaunchTimer timer(t, tp::KK_APPEND);
-            cudaError_t e = tp::launch_append_tokens(t->cfg.head_dim, a, t->stream);
-            if (e != cudaSuccess) st = cuda_fail(t, e, "token append kernel");
-        }
-        if (st != TP_OK) {
-            tp::append_tokens_unplan(t, nodes, n);
-            return st;
-        }
-    }
+    const uint64_t before = t->version;
     tp::append_tokens_commit(t, nodes, n, need);
+    if (!t->cfg.pool) return TP_OK;
+    // one launch: the tokens into their slots, and what changes in the cached
+    // decode schedule of the same leaves
+    bool patch = false;
+    const int32_t n_pairs = tp::step_patch(t, nodes, n, need == 0, before, &patch);
+    std::vector<int32_t>& w = t->scratch.step_words;  // pool slots | patch pairs
+    w.assign(t->tok_slots.begin(), t->tok_slots.end());
+    if (n_pairs > 0) w.insert(w.end(), t->patch_words.begin(), t->patch_words.begin() + 2 * (int64_t)n_pairs);
+    tp::StepWords words;
+    st = tp::step_words(t, w, &words);
+    if (st == TP_OK) {
+        tp::AppendTokensArgs a;
+        a.k = K;
+        a.v = V;
+        a.words = nullptr;
+        a.sched = t->d_sched;
+        a.pool = (uint8_t*)t->cfg.pool;
+        a.head_bytes = t->cfg.block_tokens * t->cfg.head_dim * 2;
+        a.block_bytes = (int64_t)2 * t->cfg.num_kv_heads * a.head_bytes;
+        a.hkv = t->cfg.num_kv_heads;
+        a.n = n;
+        a.n_pairs = n_pairs;
+        a.err = t->d_err;
+        a.pool_blocks = t->cfg.pool_blocks;
+        a.sched_words = (int64_t)t->sched.words.size();
+        tp::LaunchTimer timer(t, tp::KK_APPEND);
+        cudaError_t e = tp::launch_append_tokens(t->cfg.head_dim, a, words, t->stream);
+        if (e != cudaSuccess) st = cuda_fail(t, e, "token append kernel");
+    }
+    if (st != TP_OK) {  // back to the state before the call; a schedule patched on the host only is rebuilt
+        for (int32_t i = 0; i < n; ++i) --t->nodes[(size_t)nodes[i]].n_tokens;
+        tp::append_tokens_unplan(t, nodes, n);
+        --t->version;
+        if (need > 0) --t->struct_version;
+        if (patch) t->sched_valid = false;
+        return st;
+    }
+    if (patch) t->sched_version = t->version;
     return TP_OK;
 }
 
@@ -634,6 +661,7 @@ tp_status tp_decode_ex(tp_tree* t, const tp_node* leaves, int32_t n, const void*
         t->sched_flags = key_flags;
         t->sched_leaves.assign(leaves, leaves + n);
     }
+    t->sched_stream = t->stream;
     return run_schedule(t, S, Q, O, LSE);
 }
 

@@ -195,19 +195,34 @@ struct GatherArgs {
     int64_t pool_blocks = 0;  // and the pool size
 };
 
-// One token per listed node: row i of k / v goes to pool slot slots[i]
-// (block * block_tokens + row).
+// Host words of a launch (pool slots, node ids, schedule patches): up to
+// kParamWords travel as a kernel parameter (two sizes, so a small launch
+// carries a small one), more through a device buffer.
+constexpr int64_t kParamWordsSmall = 512;
+constexpr int64_t kParamWords = 4096;
+struct StepWords {
+    const int32_t* host = nullptr;    // used when n <= kParamWords
+    const int32_t* device = nullptr;  // the same words on the device otherwise
+    int64_t n = 0;
+};
+
+// One token per listed node: row i of k / v goes to pool slot words[i]
+// (block * block_tokens + row); then sched[words[n + 2k]] = words[n + 2k + 1]
+// for the n_pairs words of the cached decode schedule that change with it.
 struct AppendTokensArgs {
     const void* k;
     const void* v;
-    const int32_t* slots;
+    const int32_t* words;  // set by the launcher
+    int32_t* sched;
     uint8_t* pool;
     int64_t block_bytes;
     int32_t head_bytes;
     int32_t hkv;
     int32_t n;
-    int32_t* err = nullptr;   // bounds-checked build: device error word
-    int64_t pool_blocks = 0;  // and the pool size the slots are checked against
+    int32_t n_pairs;
+    int32_t* err = nullptr;   // bounds-checked build: device error word,
+    int64_t pool_blocks = 0;  // the pool size the slots are checked against
+    int64_t sched_words = 0;  // and the schedule length the patches are
 };
 
 // Synthetic activations of the stand-in model (splitmix.h): row i is token
@@ -230,9 +245,8 @@ struct SynthArgs {
 // stand-in activations of each row's new token, K and V written straight
 // into the row's pool slot, Q into q; then the decode schedule's patches.
 struct StepArgs {
-    const int32_t* row_node;  // [n] node of each row
-    const int32_t* slots;     // [n] pool slot of each row's new token
-    const int32_t* pairs;     // [2 n_pairs]: (schedule word index, new value)
+    const int32_t* words;  // [n] node of each row | [n] pool slot of its new token | [2 n_pairs]
+                           // (schedule word index, new value); set by the launcher
     int32_t* sched;
     uint8_t* pool;
     uint16_t* q;              // [n][q_width]
@@ -268,12 +282,12 @@ cudaError_t launch_merge(int head_dim, const MergeArgs& a, cudaStream_t s);
 cudaError_t launch_gather(int head_dim, const GatherArgs& a, int64_t n_tokens, cudaStream_t s);
 // sched[pairs[2k]] = pairs[2k + 1] for k < n (sched_words and err: the
 // bounds-checked build's limit and error word).
-cudaError_t launch_patch(int32_t* sched, const int32_t* pairs, int32_t n, cudaStream_t s, int64_t sched_words = 0,
+cudaError_t launch_patch(int32_t* sched, const StepWords& pairs, int32_t n, cudaStream_t s, int64_t sched_words = 0,
                          int32_t* err = nullptr);
 cudaError_t launch_wait_probe(int32_t* err, uint64_t limit_ns, cudaStream_t s);
-cudaError_t launch_append_tokens(int head_dim, const AppendTokensArgs& a, cudaStream_t s);
+cudaError_t launch_append_tokens(int head_dim, const AppendTokensArgs& a, const StepWords& w, cudaStream_t s);
 cudaError_t launch_synth(const SynthArgs& a, cudaStream_t s);
-cudaError_t launch_rollout_step(int head_dim, const StepArgs& a, cudaStream_t s);
+cudaError_t launch_rollout_step(int head_dim, const StepArgs& a, const StepWords& w, cudaStream_t s);
 cudaError_t launch_advantage(const AdvantageArgs& a, cudaStream_t s);
 int decode_smem_bytes(int head_dim);
 // Device address of the library's static scratch array (tp_decode_noalloc).
@@ -341,7 +355,7 @@ struct SchedScratch {
     std::vector<int32_t> units[3], sorted, bucket;
     std::vector<int32_t> pair_occ, pair_slot, merge_off, merge_pos, merge_slot;
     std::vector<int32_t> tile_pos, node_tile_off, vis;  // prefill
-    std::vector<int32_t> step_words;                    // rollout_token_step's upload
+    std::vector<int32_t> step_words;                    // words of a token step's launch
 };
 
 }  // namespace tp
@@ -420,14 +434,14 @@ struct tp_tree {
     bool sched_valid = false;
     uint64_t sched_version = 0;
     uint64_t sched_struct = 0;  // struct_version the cached schedule was built at
+    cudaStream_t sched_stream = nullptr;  // stream of the last attention that read it
     std::vector<int32_t> patch_words;
-    int32_t* d_patch = nullptr;
-    int64_t d_patch_cap = 0;
 
-    // tp_append_tokens: pool slot of each appended token
+    // tp_append_tokens: pool slot of each appended token; device words of
+    // launches with more than a kernel parameter holds
     std::vector<int32_t> tok_slots;
-    int32_t* d_tok_slots = nullptr;
-    int64_t d_tok_slots_cap = 0;
+    int32_t* d_step = nullptr;
+    int64_t d_step_cap = 0;
     uint32_t sched_flags = 0;
     std::vector<int32_t> sched_leaves;
 };
@@ -462,8 +476,18 @@ tp_status stage_upload(tp_tree* t, int32_t* dst, const int32_t* src, int64_t wor
 tp_status append_tokens_plan(tp_tree* t, const tp_node* nodes, int32_t n, int64_t* need);
 void append_tokens_unplan(tp_tree* t, const tp_node* nodes, int32_t n);
 void append_tokens_commit(tp_tree* t, const tp_node* nodes, int32_t n, int64_t need);
-tp_status rollout_token_step(tp_tree* t, const tp_node* nodes, int32_t n, int32_t* d_buf, int64_t buf_words,
-                             uint64_t seed, int32_t pos, uint16_t* q, uint32_t decode_flags);
+// The cached decode schedule's words that change with one more token on each
+// of nodes (already counted) into t->patch_words, when that schedule is the
+// one for exactly these nodes and the tokens stay inside their last blocks
+// (`stays`, `before`: the tree's version before the append) and its last
+// reader ran on the stream the tree has now; 0 otherwise.
+// The caller's launch applies them; *patched says that the schedule is then
+// current.
+int32_t step_patch(tp_tree* t, const tp_node* nodes, int32_t n, bool stays, uint64_t before, bool* patched);
+// The words of a launch: as they are, or uploaded when they are too many.
+tp_status step_words(tp_tree* t, const std::vector<int32_t>& words, StepWords* out);
+tp_status rollout_token_step(tp_tree* t, const tp_node* nodes, int32_t n, uint64_t seed, int32_t pos, uint16_t* q,
+                             uint32_t decode_flags);
 
 // forest.cpp
 tp_status fail(tp_tree* t, tp_status code, const std::string& msg);

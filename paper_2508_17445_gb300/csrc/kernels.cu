@@ -295,26 +295,55 @@ __global__ void append_kernel(const AppendArgs a) {
     }
 }
 
+// -------------------------------------------------------- token-step words --
+// The host words of a token step (row nodes, pool slots, schedule patches)
+// travel with the launch. Bound by launches and their gaps: an upload costs
+// the host an event wait, a copy and a record and the stream one more
+// operation in front of each kernel.
+template <int CAP>
+struct ParamWords {
+    int32_t v[CAP];
+};
+
+template <int CAP>  // CAP == 1: the words are on the device
+__device__ __forceinline__ int32_t step_word(const ParamWords<CAP>& p, const int32_t* words, int64_t k) {
+    return CAP == 1 ? words[k] : p.v[k];
+}
+
+// Schedule patches: pair k of the list that starts at word `at`.
+template <int CAP>
+__device__ __forceinline__ void patch_word(const ParamWords<CAP>& p, const int32_t* words, int64_t at, int64_t k,
+                                           int32_t* sched, int64_t sched_words, int32_t* err) {
+    const int32_t w = step_word(p, words, at + 2 * k);
+    if (check(in_range(w, sched_words), err)) sched[w] = step_word(p, words, at + 2 * k + 1);
+}
+
 // ----------------------------------------------------------- token append --
-// Decode-loop append: one token for each of n nodes, each to its own slot.
-template <int HD>
-__global__ void append_tokens_kernel(const AppendTokensArgs a) {
+// Decode-loop append: one token for each of n nodes, each to its own slot;
+// then the cached schedule's patches. One block per row (grid-stride), one
+// thread per 16-byte chunk.
+constexpr int kTokenThreads = 128;
+
+template <int HD, int CAP>
+__global__ void __launch_bounds__(kTokenThreads)
+    append_tokens_kernel(const AppendTokensArgs a, const __grid_constant__ ParamWords<CAP> p) {
     constexpr int CH = HD / 8;
-    const int64_t per_kv = (int64_t)a.n * a.hkv * CH;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < 2 * per_kv;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int kv = idx >= per_kv;
-        const int64_t r = kv ? idx - per_kv : idx;
-        const int c = (int)(r % CH);
-        const int h = (int)((r / CH) % a.hkv);
-        const int i = (int)(r / ((int64_t)CH * a.hkv));
-        const int32_t slot = a.slots[i];
+    const int per_row = a.hkv * CH;
+    for (int i = blockIdx.x; i < a.n; i += gridDim.x) {
+        const int32_t slot = step_word(p, a.words, i);
         if (!check(in_range(slot, a.pool_blocks * kBlockTokens), a.err)) continue;
-        const uint4 val = reinterpret_cast<const uint4*>(kv ? a.v : a.k)[r];
-        uint8_t* dst = a.pool + (int64_t)(slot / kBlockTokens) * a.block_bytes +
-                       (int64_t)(kv * a.hkv + h) * a.head_bytes + kv_off<kBlockTokens>(slot % kBlockTokens, c);
-        *reinterpret_cast<uint4*>(dst) = val;
+        uint8_t* dst = a.pool + (int64_t)(slot / kBlockTokens) * a.block_bytes;
+        const int row = slot % kBlockTokens;
+        for (int r = threadIdx.x; r < 2 * per_row; r += kTokenThreads) {
+            const int kv = r >= per_row, rr = kv ? r - per_row : r;
+            const uint4 val = reinterpret_cast<const uint4*>(kv ? a.v : a.k)[(int64_t)i * per_row + rr];
+            *reinterpret_cast<uint4*>(dst + (int64_t)(kv * a.hkv + rr / CH) * a.head_bytes +
+                                      kv_off<kBlockTokens>(row, rr % CH)) = val;
+        }
     }
+    for (int64_t k = (int64_t)blockIdx.x * kTokenThreads + threadIdx.x; k < a.n_pairs;
+         k += (int64_t)gridDim.x * kTokenThreads)
+        patch_word(p, a.words, a.n, k, a.sched, a.sched_words, a.err);
 }
 
 // ------------------------------------------------------ stand-in activations --
@@ -362,41 +391,41 @@ __global__ void synth_kernel(const SynthArgs a) {
 // append_tokens_kernel would write), Q into q; then the schedule words the
 // append changed are patched. One thread per 16-byte K/V chunk (two draws),
 // per Q draw, per patch.
-template <int HD>
-__global__ void rollout_step_kernel(const StepArgs a) {
+// Row i is blockIdx.x (grid-stride), blockIdx.y splits the row's items.
+constexpr int kStepThreads = 256;
+
+template <int HD, int CAP>
+__global__ void __launch_bounds__(kStepThreads)
+    rollout_step_kernel(const StepArgs a, const __grid_constant__ ParamWords<CAP> p) {
     constexpr int CH = HD / 8;
-    const int64_t kv_items = (int64_t)a.n * 2 * a.hkv * CH;
-    const int q_words = a.q_width / 4;
-    const int64_t q_items = (int64_t)a.n * q_words;
-    const int64_t total = kv_items + q_items + a.n_pairs;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        if (idx < kv_items) {
-            const int c = (int)(idx % CH);
-            const int h = (int)((idx / CH) % a.hkv);
-            const int kv = (int)((idx / ((int64_t)CH * a.hkv)) & 1);
-            const int i = (int)(idx / ((int64_t)CH * a.hkv * 2));
-            const uint32_t node = (uint32_t)a.row_node[i], tag = kv ? kTagV : kTagK;
-            const uint32_t w0 = (uint32_t)(h * (HD / 4) + 2 * c);  // the chunk's two draws of the row
-            const uint2 x0 = synth_words(splitmix64(a.seed, draw_counter(tag, node, (uint32_t)a.pos, w0)));
-            const uint2 x1 = synth_words(splitmix64(a.seed, draw_counter(tag, node, (uint32_t)a.pos, w0 + 1)));
-            const int32_t slot = a.slots[i];
-            if (!check(in_range(slot, a.pool_blocks * kBlockTokens), a.err)) continue;
-            uint8_t* dst = a.pool + (int64_t)(slot / kBlockTokens) * a.block_bytes +
-                           (int64_t)(kv * a.hkv + h) * a.head_bytes + kv_off<kBlockTokens>(slot % kBlockTokens, c);
-            *reinterpret_cast<uint4*>(dst) = make_uint4(x0.x, x0.y, x1.x, x1.y);
-        } else if (idx < kv_items + q_items) {
-            const int64_t r = idx - kv_items;
-            const int i = (int)(r / q_words), w = (int)(r % q_words);
-            const uint32_t node = (uint32_t)a.row_node[i];
-            *reinterpret_cast<uint2*>(a.q + (int64_t)i * a.q_width + 4 * w) =
-                synth_words(splitmix64(a.seed, draw_counter(kTagQ, node, (uint32_t)a.pos, (uint32_t)w)));
-        } else {
-            const int64_t k = idx - kv_items - q_items;
-            if (!check(in_range(a.pairs[2 * k], a.sched_words), a.err)) continue;
-            a.sched[a.pairs[2 * k]] = a.pairs[2 * k + 1];
+    const int kv_items = 2 * a.hkv * CH, items = kv_items + a.q_width / 4;
+    const int t0 = blockIdx.y * kStepThreads + threadIdx.x, step = gridDim.y * kStepThreads;
+    for (int i = blockIdx.x; i < a.n; i += gridDim.x) {
+        const uint32_t node = (uint32_t)step_word(p, a.words, i);
+        const int32_t slot = step_word(p, a.words, (int64_t)a.n + i);
+        const bool slot_ok = check(in_range(slot, a.pool_blocks * kBlockTokens), a.err);
+        uint8_t* block = a.pool + (int64_t)(slot / kBlockTokens) * a.block_bytes;
+        for (int idx = t0; idx < items; idx += step) {
+            if (idx < kv_items) {
+                const int c = idx % CH, head = idx / CH;  // head: kv * hkv + kv head
+                const int kv = head >= a.hkv, h = kv ? head - a.hkv : head;
+                const uint32_t tag = kv ? kTagV : kTagK;
+                const uint32_t w0 = (uint32_t)(h * (HD / 4) + 2 * c);  // the chunk's two draws of the row
+                const uint2 x0 = synth_words(splitmix64(a.seed, draw_counter(tag, node, (uint32_t)a.pos, w0)));
+                const uint2 x1 = synth_words(splitmix64(a.seed, draw_counter(tag, node, (uint32_t)a.pos, w0 + 1)));
+                if (!slot_ok) continue;
+                *reinterpret_cast<uint4*>(block + (int64_t)head * a.head_bytes +
+                                          kv_off<kBlockTokens>(slot % kBlockTokens, c)) =
+                    make_uint4(x0.x, x0.y, x1.x, x1.y);
+            } else {
+                const int w = idx - kv_items;
+                *reinterpret_cast<uint2*>(a.q + (int64_t)i * a.q_width + 4 * w) =
+                    synth_words(splitmix64(a.seed, draw_counter(kTagQ, node, (uint32_t)a.pos, (uint32_t)w)));
+            }
         }
     }
+    for (int64_t k = (int64_t)blockIdx.x * step + t0; k < a.n_pairs; k += (int64_t)gridDim.x * step)
+        patch_word(p, a.words, 2ll * a.n, k, a.sched, a.sched_words, a.err);
 }
 
 // -------------------------------------------------------- tree advantage --
@@ -573,9 +602,11 @@ __global__ void __launch_bounds__(kAdvAbarThreads) advantage_abar_kernel(const A
 }
 
 // ------------------------------------------------------- schedule patch --
-__global__ void patch_kernel(int32_t* sched, const int32_t* pairs, int32_t n, int64_t sched_words, int32_t* err) {
+template <int CAP>
+__global__ void patch_kernel(int32_t* sched, const __grid_constant__ ParamWords<CAP> p, const int32_t* words, int32_t n,
+                             int64_t sched_words, int32_t* err) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n && check(in_range(pairs[2 * k], sched_words), err)) sched[pairs[2 * k]] = pairs[2 * k + 1];
+    if (k < n) patch_word(p, words, 0, k, sched, sched_words, err);
 }
 
 // ------------------------------------------------------------------ gather --
@@ -2443,31 +2474,57 @@ cudaError_t launch_wait_probe(int32_t* err, uint64_t limit_ns, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_patch(int32_t* sched, const int32_t* pairs, int32_t n, cudaStream_t s, int64_t sched_words,
+// Calls launch(ParamWords, device words) with the words in the smallest
+// parameter that holds them: 2 KB, 16 KB, or the device copy.
+namespace {
+template <typename Launch>
+cudaError_t with_words(const StepWords& w, Launch launch) {
+    if (w.n <= kParamWordsSmall) {
+        ParamWords<kParamWordsSmall> p;
+        std::copy(w.host, w.host + w.n, p.v);
+        launch(p, (const int32_t*)nullptr);
+    } else if (w.n <= kParamWords) {
+        ParamWords<kParamWords> p;
+        std::copy(w.host, w.host + w.n, p.v);
+        launch(p, (const int32_t*)nullptr);
+    } else {
+        launch(ParamWords<1>{}, w.device);
+    }
+    return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_patch(int32_t* sched, const StepWords& pairs, int32_t n, cudaStream_t s, int64_t sched_words,
                          int32_t* err) {
-    patch_kernel<<<(n + 255) / 256, 256, 0, s>>>(sched, pairs, n, sched_words, err);
-    return cudaGetLastError();
+    return with_words(pairs, [&](const auto& p, const int32_t* words) {
+        patch_kernel<<<(n + 255) / 256, 256, 0, s>>>(sched, p, words, n, sched_words, err);
+    });
 }
 
-cudaError_t launch_append_tokens(int hd, const AppendTokensArgs& a, cudaStream_t s) {
-    const int64_t chunks = 2ll * a.n * a.hkv * (hd / 8);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((chunks + 255) / 256, 152 * 16));
-    if (hd == 64)
-        append_tokens_kernel<64><<<grid, 256, 0, s>>>(a);
-    else
-        append_tokens_kernel<128><<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_append_tokens(int hd, const AppendTokensArgs& a0, const StepWords& w, cudaStream_t s) {
+    const int grid = std::min(std::max(a0.n, 1), 152 * 16);
+    return with_words(w, [&](const auto& p, const int32_t* words) {
+        AppendTokensArgs a = a0;
+        a.words = words;
+        if (hd == 64)
+            append_tokens_kernel<64><<<grid, kTokenThreads, 0, s>>>(a, p);
+        else
+            append_tokens_kernel<128><<<grid, kTokenThreads, 0, s>>>(a, p);
+    });
 }
 
-cudaError_t launch_rollout_step(int hd, const StepArgs& a, cudaStream_t s) {
-    const int64_t items = (int64_t)a.n * (2 * a.hkv * (hd / 8) + a.q_width / 4) + a.n_pairs;
-    if (items == 0) return cudaSuccess;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((items + 255) / 256, 152 * 16));
-    if (hd == 64)
-        rollout_step_kernel<64><<<grid, 256, 0, s>>>(a);
-    else
-        rollout_step_kernel<128><<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_rollout_step(int hd, const StepArgs& a0, const StepWords& w, cudaStream_t s) {
+    if (a0.n == 0) return cudaSuccess;
+    const int items = 2 * a0.hkv * (hd / 8) + a0.q_width / 4;
+    const dim3 grid(std::min(a0.n, 152 * 16), std::min((items + kStepThreads - 1) / kStepThreads, 8));
+    return with_words(w, [&](const auto& p, const int32_t* words) {
+        StepArgs a = a0;
+        a.words = words;
+        if (hd == 64)
+            rollout_step_kernel<64><<<grid, kStepThreads, 0, s>>>(a, p);
+        else
+            rollout_step_kernel<128><<<grid, kStepThreads, 0, s>>>(a, p);
+    });
 }
 
 cudaError_t launch_synth(const SynthArgs& a, cudaStream_t s) {

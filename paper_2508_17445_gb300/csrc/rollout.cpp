@@ -111,7 +111,7 @@ class Rollout {
         : t_(t), p_(p), ev_(ev), cap_(cap), probe_(probe) {}
     ~Rollout() {
         if (t_->cfg.pool) cudaStreamSynchronize(t_->stream);
-        for (DevBuf* b : {&k_, &v_, &q_, &o_, &lse_, &rows_})
+        for (DevBuf* b : {&k_, &v_, &q_, &o_, &lse_})
             if (b->p) cudaFree(b->p);
     }
     tp_status run(tp_rollout_stats* stats);
@@ -127,7 +127,7 @@ class Rollout {
     std::vector<QueryState> qs_;
     std::vector<Path> queue_;
     std::vector<Segment> seg_;
-    DevBuf k_, v_, q_, o_, lse_, rows_;
+    DevBuf k_, v_, q_, o_, lse_;
     std::vector<int32_t> gen_, counts_;
     std::vector<double> frac_, logp_;
     std::vector<int32_t> order_, split_;
@@ -220,9 +220,8 @@ tp_status Rollout::decode_tokens() {
             if (seg_[i].len > t) gen_.push_back(queue_[i].node);
         const int32_t n = (int32_t)gen_.size();
         // the token's stand-in activations straight into the pool, Q into q_,
-        // and the cached decode schedule patched: one upload, one launch
-        tp_status s = tp::rollout_token_step(t_, gen_.data(), n, (int32_t*)rows_.p, rows_.cap / 4, p_.seed, t,
-                                             (uint16_t*)q_.p, p_.decode_flags);
+        // and the cached decode schedule patched: one launch
+        tp_status s = tp::rollout_token_step(t_, gen_.data(), n, p_.seed, t, (uint16_t*)q_.p, p_.decode_flags);
         if (s != TP_OK) return s;
         note_pool();
         s = tp_decode_ex(t_, gen_.data(), n, q_.p, o_.p, (float*)lse_.p, p_.decode_flags);
@@ -284,7 +283,6 @@ tp_status Rollout::run(tp_rollout_stats* stats) {
         if (s == TP_OK && p.decode) s = grow(q_, rows_max * qw * 2, "rollout Q");
         if (s == TP_OK && p.decode) s = grow(o_, rows_max * qw * 2, "rollout O");
         if (s == TP_OK && p.decode) s = grow(lse_, rows_max * t_->cfg.num_q_heads * 4, "rollout LSE");
-        if (s == TP_OK && p.decode) s = grow(rows_, rows_max * 16, "rollout token-step words");
         if (s != TP_OK) return s;
     }
     qs_.assign((size_t)nq, QueryState());
