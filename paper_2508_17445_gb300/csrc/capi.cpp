@@ -355,9 +355,6 @@ tp_status tp_tree_destroy(tp_tree* t) {
     if (t->d_gather_tiles) cudaFree(t->d_gather_tiles);
     if (t->d_step) cudaFree(t->d_step);
     for (cudaEvent_t e : t->ev_pool) cudaEventDestroy(e);
-    if (t->ev_fork) cudaEventDestroy(t->ev_fork);
-    if (t->ev_join) cudaEventDestroy(t->ev_join);
-    if (t->side) cudaStreamDestroy(t->side);
     for (int k = 0; k < 2; ++k) {
         if (t->h_pinned[k]) cudaFreeHost(t->h_pinned[k]);
         if (t->h_pinned_ev[k]) cudaEventDestroy(t->h_pinned_ev[k]);
@@ -866,15 +863,9 @@ tp_status run_schedule(tp_tree* t, const tp::Schedule& S, const void* Q, void* O
     a.kv_read_once = S.kv_read_once ? 1 : 0;
     a.ext = extents_of(t, S);
     cudaError_t e = cudaSuccess;
-    if (S.n_tc > 0 && S.n_units > S.n_tc && !t->side) {  // concurrent tcgen05 units need a second stream
-        e = cudaStreamCreateWithFlags(&t->side, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->ev_fork, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->ev_join, cudaEventDisableTiming);
-        if (e != cudaSuccess) return cuda_fail(t, e, "side stream");
-    }
     if (a.n_units > 0) {
         tp::LaunchTimer timer(t, tp::KK_DECODE);
-        e = tp::launch_decode(hd, a, t->stream, t->side, t->ev_fork, t->ev_join);
+        e = tp::launch_decode(hd, a, t->stream);
         timer.kernels((S.n_tc > 0) + (S.n_tensor > 0) + (S.n_units > S.n_tc + S.n_tensor));
     }
     if (e != cudaSuccess) return cuda_fail(t, e, "decode kernel");

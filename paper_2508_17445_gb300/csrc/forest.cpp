@@ -288,8 +288,7 @@ tp_status build_schedule(tp_tree* t, const tp_node* leaves, int32_t n, uint32_t 
     // TP_MMA_SYNC; TP_DECODE_TCGEN05 alone keeps it to long, tall chunks. A
     // call reading less than kSmallCallBytes of K/V is bound by launch
     // latency: its stacked rows stay on mma.sync, so the whole call is one
-    // attention kernel on the tree's stream, without the tcgen05 kernel's
-    // side-stream fork and join (TP_DECODE_ALL_TCGEN05 still forces tcgen05).
+    // attention kernel (TP_DECODE_ALL_TCGEN05 still forces tcgen05).
     const int64_t tile_bytes = (int64_t)t->cfg.block_tokens * t->cfg.head_dim * 2 * 2;
     const bool small_call = work * tile_bytes < kSmallCallBytes && !(flags & TP_DECODE_ALL_TCGEN05);
     const bool use_tc = (flags & TP_MMA_SYNC) == 0 && !small_call;

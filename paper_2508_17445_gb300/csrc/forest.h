@@ -42,7 +42,7 @@ constexpr int kTcMinTiles = 32;
 constexpr int kTcAnyRows = 17;
 constexpr int kTcRowsPerUnit = 128;
 // Decode calls reading less K/V than this (about a microsecond of HBM time)
-// keep every unit on mma.sync: one attention kernel, no side stream.
+// keep every unit on mma.sync: one attention kernel.
 constexpr int64_t kSmallCallBytes = 1 << 20;
 // Longest unit in pool blocks (the decode kernel keeps a unit's tile words
 // in shared memory).
@@ -133,11 +133,12 @@ struct DecodeArgs {
     const int32_t* unit_pos = nullptr;  // prefill: path position of each unit's first token
     uint16_t* out = nullptr;            // units with slot_base < 0 write O (bf16 [n][Hq][hd]) and
     float* out_lse = nullptr;           // LSE (natural log) here directly: their rows have no other part
-    int32_t* counters;    // [3] next unit per kind (0 at launch; the merge re-arms them)
+    int32_t* counters;    // [3] units claimed per kind past each CTA's first (0 at launch; the merge re-arms them)
     int32_t* counter;     // the counter of the launch in flight (set by the launcher)
     int32_t n_tc_units;      // units [0, n_tc) are tcgen05 units,
     int32_t n_tensor_units;  // then n_tensor mma.sync units, then CUDA-core units
     int32_t unit_begin, unit_end;  // unit range of the launch in flight
+    int32_t late_wait = 0;  // the launch runs beside its predecessor on the stream and waits for it last
     int64_t block_bytes;  // bytes of one pool block (K and V, all kv heads)
     int32_t head_bytes;   // bytes of one (block, K|V, kv head) tile
     int32_t n_units;
@@ -273,11 +274,7 @@ int64_t advantage_ws_bytes(int64_t n_nodes, int64_t n_out);
 
 // Launchers (kernels.cu). Return cudaSuccess or the launch error.
 cudaError_t launch_append(int head_dim, const AppendArgs& a, cudaStream_t s);
-// With side != nullptr and both tcgen05 and other units present, the
-// tcgen05 units run on `side` concurrently with the rest (fork/join through
-// the two events), so a small tcgen05 launch does not leave SMs idle.
-cudaError_t launch_decode(int head_dim, const DecodeArgs& a, cudaStream_t s, cudaStream_t side = nullptr,
-                          cudaEvent_t fork = nullptr, cudaEvent_t join = nullptr);
+cudaError_t launch_decode(int head_dim, const DecodeArgs& a, cudaStream_t s);
 cudaError_t launch_merge(int head_dim, const MergeArgs& a, cudaStream_t s);
 cudaError_t launch_gather(int head_dim, const GatherArgs& a, int64_t n_tokens, cudaStream_t s);
 // sched[pairs[2k]] = pairs[2k + 1] for k < n (sched_words and err: the
@@ -386,9 +383,6 @@ struct tp_tree {
     int pinned_next = 0;
     int32_t* d_gather_tiles = nullptr;
     int64_t d_gather_cap = 0;
-    cudaStream_t side = nullptr;  // second stream for concurrent tcgen05 units
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-
     // prefill schedules (rebuilt every call): two device buffers used in
     // turn, uploaded on a copy stream of their own once the kernels that read
     // the buffer two calls back are done, so a call's upload overlaps the

@@ -32,6 +32,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <utility>
 
 #include "forest.h"
 #include "splitmix.h"
@@ -260,6 +261,20 @@ __device__ __forceinline__ int kv_off(int row, int chunk) {
     return (chunk >> 3) * (ROWS * 128) + row * 128 + (((chunk & 7) ^ (row & 7)) << 4);
 }
 
+// Programmatic dependent launch. Kernels of a call are launched while their
+// predecessor on the stream still runs: each sets itself up, then waits
+// (dep_wait) until the predecessor has completed and its writes are visible,
+// and lets its own successor start (dep_trigger). A kernel that reads nothing
+// of its predecessor may wait last instead, so that its completion still
+// means that everything before it has completed. What it hides is the launch,
+// the CTA set-up and the first schedule reads of each of a call's two or three
+// kernels: against plain launches on two streams, small and mid-size calls
+// lose 4-7 us (8 leaves of 200 tokens 12.7 -> 7.6 us, one 8k path 15.4 -> 10.4,
+// 16 leaves of 2.7k 25.2 -> 17.7, 32 diverging 8k paths 62 -> 53.5, a rollout
+// batch's token step 32 -> 23); calls of a GB and more stay within 1-5%.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Bounds-checked build: true when an index check passed; otherwise records
 // the failure in the device error word (the caller skips the access). In the
 // default build it is `true` and the check compiles away.
@@ -328,6 +343,8 @@ template <int HD, int CAP>
 __global__ void __launch_bounds__(kTokenThreads)
     append_tokens_kernel(const AppendTokensArgs a, const __grid_constant__ ParamWords<CAP> p) {
     constexpr int CH = HD / 8;
+    dep_trigger();
+    dep_wait();
     const int per_row = a.hkv * CH;
     for (int i = blockIdx.x; i < a.n; i += gridDim.x) {
         const int32_t slot = step_word(p, a.words, i);
@@ -398,6 +415,8 @@ template <int HD, int CAP>
 __global__ void __launch_bounds__(kStepThreads)
     rollout_step_kernel(const StepArgs a, const __grid_constant__ ParamWords<CAP> p) {
     constexpr int CH = HD / 8;
+    dep_trigger();
+    dep_wait();
     const int kv_items = 2 * a.hkv * CH, items = kv_items + a.q_width / 4;
     const int t0 = blockIdx.y * kStepThreads + threadIdx.x, step = gridDim.y * kStepThreads;
     for (int i = blockIdx.x; i < a.n; i += gridDim.x) {
@@ -605,6 +624,8 @@ __global__ void __launch_bounds__(kAdvAbarThreads) advantage_abar_kernel(const A
 template <int CAP>
 __global__ void patch_kernel(int32_t* sched, const __grid_constant__ ParamWords<CAP> p, const int32_t* words, int32_t n,
                              int64_t sched_words, int32_t* err) {
+    dep_trigger();
+    dep_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n) patch_word(p, words, 0, k, sched, sched_words, err);
 }
@@ -1265,6 +1286,15 @@ struct TensorPath {
     }
 };
 
+// This CTA's k-th unit: its own index first (no round trip to the counter),
+// then whichever is next. CTAs that start beside another kernel do so one by
+// one, so their first unit comes from the counter too: assigned by index, a
+// late CTA would hold one of the longest units.
+__device__ __forceinline__ int claim_unit(const DecodeArgs& a, int k) {
+    if (a.late_wait) return a.unit_begin + atomicAdd(a.counter, 1);
+    return a.unit_begin + (int)(k == 0 ? blockIdx.x : gridDim.x + atomicAdd(a.counter, 1));
+}
+
 // Fetcher warp: claim units, publish descriptor + tile words, stage a tensor
 // unit's query rows (one bulk copy per leaf occurrence group, lanes in
 // parallel).
@@ -1278,11 +1308,11 @@ __device__ void fetch_units(const DecodeArgs& a, Ctl& c, uint8_t* qbuf) {
         if (!mbar_wait(smem_u32(&c.uempty[q]), ((k >> 1) & 1) ^ 1)) note_timeout(a, c, 2);
         int u = -1;
         if (lane == 0) {
-            u = *abort ? -1 : a.unit_begin + atomicAdd(a.counter, 1);
+            u = *abort ? -1 : claim_unit(a, k);
             if (u >= a.unit_end) u = -1;
         }
         u = __shfl_sync(0xffffffffu, u, 0);
-        const int word = (u >= 0 && lane < kUnitWords) ? a.units[(int64_t)u * kUnitWords + lane] : 0;
+        const int word = (u >= 0 && lane < kUnitWords) ? __ldcg(a.units + (int64_t)u * kUnitWords + lane) : 0;
         UnitDesc d;
         d.tile_off = __shfl_sync(0xffffffffu, word, U_TILE_OFF);
         d.n_tiles = __shfl_sync(0xffffffffu, word, U_N_TILES);
@@ -1300,7 +1330,7 @@ __device__ void fetch_units(const DecodeArgs& a, Ctl& c, uint8_t* qbuf) {
             u = -1;
         }
         if (u >= 0)
-            for (int t = lane; t < d.n_tiles; t += 32) c.tiles[q][t] = a.tiles[d.tile_off + t];
+            for (int t = lane; t < d.n_tiles; t += 32) c.tiles[q][t] = __ldcg(a.tiles + d.tile_off + t);
         if (lane == 0) {
             volatile int* dw = c.desc[q];
             dw[U_TILE_OFF] = d.tile_off;
@@ -1327,7 +1357,7 @@ __device__ void fetch_units(const DecodeArgs& a, Ctl& c, uint8_t* qbuf) {
             const int g = a.group;
             for (int r = lane; r < d.n_rows; r += 32) {  // one 2*HD-byte copy per row
                 const int item_row = d.row0 + r;
-                int occ = a.occ[d.occ_off + item_row / g];
+                int occ = __ldcg(a.occ + d.occ_off + item_row / g);
                 if (!check(in_range(occ, a.ext.n), a.err)) occ = 0;
                 const uint16_t* src = a.q + ((int64_t)occ * a.hq + d.kvh * g + item_row % g) * HD;
                 bulk_g2s(smem_u32(qbuf + r * Smem<HD>::kQPitch), src, HD * 2, smem_u32(&c.qfull));
@@ -1438,12 +1468,15 @@ __global__ void __launch_bounds__(kDecodeThreads, 2) decode_kernel(const DecodeA
     }
     fence_proxy_async();
     __syncthreads();
+    if (!a.late_wait) dep_wait();
+    dep_trigger();
     if (warp == kStreamerWarp) {
         if ((tid & 31) == 0) stream_units<HD>(a, ctl, ring);
         return;
     }
     if (warp == kFetcherWarp) {
         fetch_units<HD, KIND>(a, ctl, qbuf);
+        if (a.late_wait) dep_wait();
         return;
     }
     consume<HD, KIND>(a, ctl, ring, park, qbuf, cc_scratch);
@@ -1605,11 +1638,11 @@ __device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
         if (!mbar_wait(smem_u32(&c.uempty[q]), ((k >> 1) & 1) ^ 1)) note_timeout(a, c, 2);
         int u = -1;
         if (lane == 0) {
-            u = *abort ? -1 : a.unit_begin + atomicAdd(a.counter, 1);
+            u = *abort ? -1 : claim_unit(a, k);
             if (u >= a.unit_end) u = -1;
         }
         u = __shfl_sync(0xffffffffu, u, 0);
-        const int word = (u >= 0 && lane < kUnitWords) ? a.units[(int64_t)u * kUnitWords + lane] : 0;
+        const int word = (u >= 0 && lane < kUnitWords) ? __ldcg(a.units + (int64_t)u * kUnitWords + lane) : 0;
         const int n_tiles = __shfl_sync(0xffffffffu, word, U_N_TILES);
         const int tile_off = __shfl_sync(0xffffffffu, word, U_TILE_OFF);
         if constexpr (kBoundsCheck) {
@@ -1624,7 +1657,7 @@ __device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
             }
         }
         if (u >= 0)
-            for (int t = lane; t < n_tiles; t += 32) c.tiles[q][t] = a.tiles[tile_off + t];
+            for (int t = lane; t < n_tiles; t += 32) c.tiles[q][t] = __ldcg(a.tiles + tile_off + t);
         if (lane < kUnitWords) reinterpret_cast<volatile int*>(c.desc[q])[lane] = word;
         if (lane == kUnitWords)
             reinterpret_cast<volatile int*>(c.desc[q])[lane] = (u >= 0 && a.unit_pos) ? a.unit_pos[u] : 0;
@@ -1654,7 +1687,7 @@ __device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
         for (int i = 0; i < kRowsPerLane; ++i) {
             const int r = lane + 32 * i;
             const int item_row = row0 + r, p = item_row / g, hh = item_row - p * g;
-            int occ = r >= n_rows ? 0 : in_order ? occ_off + p : a.occ[occ_off + p];
+            int occ = r >= n_rows ? 0 : in_order ? occ_off + p : __ldcg(a.occ + occ_off + p);
             if (!check(in_range(occ, a.ext.n), a.err)) occ = 0;
             src_off[i] = ((int64_t)occ * a.hq + kvh * g + hh) * HD;
         }
@@ -2128,6 +2161,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) decode_tc_kernel(const DecodeAr
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (!a.late_wait) dep_wait();
+    dep_trigger();
     if (warp < kTcConsumerWarps)
         tc_consume<HD, CAUSAL>(a, ctl);
     else if (warp == kTcStreamerWarp) {
@@ -2140,6 +2175,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) decode_tc_kernel(const DecodeAr
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (a.late_wait) dep_wait();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(ctl.tmem), "r"(kTmemCols));
 }
 
@@ -2248,9 +2284,8 @@ __global__ void __launch_bounds__(WPR > 4 ? WPR * 32 : 128) merge_kernel(const M
     const int warp = threadIdx.x >> 5, part = warp % WPR;
     const int64_t row = (int64_t)blockIdx.x * (kWarps / WPR) + warp / WPR;
     const int lane = threadIdx.x & 31;
-    if (blockIdx.x == 0 && threadIdx.x < 3) a.counters[threadIdx.x] = 0;  // decode is done: re-arm its counters
+    dep_trigger();
     const bool in_grid = row < (int64_t)a.n * a.hq;
-    if (WPR == 1 && !in_grid) return;
     const int i = in_grid ? (int)(row / a.hq) : 0, qh = (int)(row % a.hq);
     float acc[DPL];
 #pragma unroll
@@ -2260,7 +2295,10 @@ __global__ void __launch_bounds__(WPR > 4 ? WPR * 32 : 128) merge_kernel(const M
     // The occurrence's merge record, in one round trip: lane k < 16 holds
     // word k ([count, slots...]).
     const int rw =
-        in_grid && a.merge_rec && lane < kMergeRecWords ? a.merge_rec[(int64_t)i * kMergeRecWords + lane] : -1;
+        in_grid && a.merge_rec && lane < kMergeRecWords ? __ldcg(a.merge_rec + (int64_t)i * kMergeRecWords + lane) : -1;
+    dep_wait();  // the attention kernels have completed (their schedule was there before they began)
+    if (blockIdx.x == 0 && threadIdx.x < 3) a.counters[threadIdx.x] = 0;  // re-arm their counters
+    if (WPR == 1 && !in_grid) return;
     const int ns_rec = __shfl_sync(0xffffffffu, rw, 0);  // -1: the CSR (more than 15 slots, or no records)
     int ns = 0;
     if (ns_rec >= 0) {
@@ -2325,6 +2363,23 @@ __global__ void __launch_bounds__(WPR > 4 ? WPR * 32 : 128) merge_kernel(const M
     if (lane == 0) a.lse[(int64_t)i * a.hq + qh] = (M + __log2f(L)) * 0.69314718055994531f;
 }
 
+// Launch that may start while its predecessor on the stream still runs (the
+// kernel waits for it with dep_wait).
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 template <int HD, int KIND>
 int decode_grid() {
     // persistent grid: every resident CTA slot of the device
@@ -2351,8 +2406,8 @@ cudaError_t launch_range(DecodeArgs a, int begin, int end, int32_t* counter, cud
     a.unit_begin = begin;
     a.unit_end = end;
     a.counter = counter;
-    decode_kernel<HD, KIND><<<std::min(end - begin, slots), kDecodeThreads, decode_smem<HD, KIND>(), s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(decode_kernel<HD, KIND>, std::min(end - begin, slots), kDecodeThreads,
+                            decode_smem<HD, KIND>(), s, a);
 }
 
 template <int HD, bool CAUSAL>
@@ -2395,34 +2450,41 @@ cudaError_t launch_tc_range(DecodeArgs a, int begin, int end, int32_t* counter, 
     a.unit_begin = begin;
     a.unit_end = end;
     a.counter = counter;
-    if (causal)
-        decode_tc_kernel<HD, true><<<std::min(end - begin, slots), kTcThreads, TcSmem<HD>::kBytes, s>>>(a);
-    else
-        decode_tc_kernel<HD, false><<<std::min(end - begin, slots), kTcThreads, TcSmem<HD>::kBytes, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(causal ? decode_tc_kernel<HD, true> : decode_tc_kernel<HD, false>,
+                            std::min(end - begin, slots), kTcThreads, TcSmem<HD>::kBytes, s, a);
 }
 
+// Both attention kernels of a call run side by side: the second is launched
+// once every CTA of the first has started (it reads nothing that the first
+// writes) and takes the CTA slots the first leaves free, so a small tcgen05
+// launch leaves no SM idle. It completes only after the first has
+// (late_wait), so what follows on the stream waits for both.
+//
+// The tcgen05 units go first, until there are about six for every resident
+// CTA: few of them end unevenly, and the mma.sync units fill those gaps, while
+// many end evenly by themselves, and launched last their partials (the larger
+// part) are still in L2 when the merge reads them. Measured, tcgen05 units
+// first against last: 16 diverging prompts (1180 units) 509 / 520 us, 64 leaves
+// x 8 prompts with a 2k prefix (1536) 309 / 317, 48 binary trees (1344) 245 /
+// 246; 24 diverging prompts (1792) 828 / 823, 64 binary trees (1792) 326 / 322,
+// 32 diverging prompts (2444) 1116 / 1101, 96 binary trees (2688) 490 / 483.
+constexpr int kTcLastUnits = 11 * 152;
+
 template <int HD>
-cudaError_t launch_decode_hd(const DecodeArgs& a, cudaStream_t s, cudaStream_t side, cudaEvent_t fork,
-                             cudaEvent_t join) {
+cudaError_t launch_decode_hd(const DecodeArgs& a, cudaStream_t s) {
     const int tc_end = a.n_tc_units, mma_end = tc_end + a.n_tensor_units;
-    cudaError_t e;
-    const bool concurrent = side && fork && join && tc_end > 0 && a.n_units > tc_end;
-    if (concurrent) {
-        if ((e = cudaEventRecord(fork, s)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess) return e;
-        if ((e = launch_tc_range<HD>(a, 0, tc_end, a.counters, side)) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(join, side)) != cudaSuccess) return e;
-    } else {
-        e = launch_tc_range<HD>(a, 0, tc_end, a.counters, s);
-    }
+    const bool tc_last = tc_end >= kTcLastUnits && mma_end > tc_end;
+    DecodeArgs first = a, second = a;
+    second.late_wait = tc_end > 0 && mma_end > tc_end;
+    cudaError_t e = cudaSuccess;
+    if (!tc_last) e = launch_tc_range<HD>(first, 0, tc_end, a.counters, s);
     if (e != cudaSuccess) return e;
-    e = a.vis ? launch_range<HD, KIND_PREFILL>(a, tc_end, mma_end, a.counters + 1, s)
-              : launch_range<HD, KIND_TENSOR>(a, tc_end, mma_end, a.counters + 1, s);
+    const DecodeArgs& m = tc_last ? first : second;
+    e = a.vis ? launch_range<HD, KIND_PREFILL>(m, tc_end, mma_end, a.counters + 1, s)
+              : launch_range<HD, KIND_TENSOR>(m, tc_end, mma_end, a.counters + 1, s);
+    if (e == cudaSuccess && tc_last) e = launch_tc_range<HD>(second, 0, tc_end, a.counters, s);
     if (e != cudaSuccess) return e;
-    e = launch_range<HD, KIND_CUDA_CORE>(a, mma_end, a.n_units, a.counters + 2, s);
-    if (e != cudaSuccess) return e;
-    return concurrent ? cudaStreamWaitEvent(s, join, 0) : cudaSuccess;
+    return launch_range<HD, KIND_CUDA_CORE>(a, mma_end, a.n_units, a.counters + 2, s);
 }
 
 }  // namespace
@@ -2482,22 +2544,22 @@ cudaError_t with_words(const StepWords& w, Launch launch) {
     if (w.n <= kParamWordsSmall) {
         ParamWords<kParamWordsSmall> p;
         std::copy(w.host, w.host + w.n, p.v);
-        launch(p, (const int32_t*)nullptr);
-    } else if (w.n <= kParamWords) {
+        return launch(p, (const int32_t*)nullptr);
+    }
+    if (w.n <= kParamWords) {
         ParamWords<kParamWords> p;
         std::copy(w.host, w.host + w.n, p.v);
-        launch(p, (const int32_t*)nullptr);
-    } else {
-        launch(ParamWords<1>{}, w.device);
+        return launch(p, (const int32_t*)nullptr);
     }
-    return cudaGetLastError();
+    return launch(ParamWords<1>{}, w.device);
 }
 }  // namespace
 
 cudaError_t launch_patch(int32_t* sched, const StepWords& pairs, int32_t n, cudaStream_t s, int64_t sched_words,
                          int32_t* err) {
     return with_words(pairs, [&](const auto& p, const int32_t* words) {
-        patch_kernel<<<(n + 255) / 256, 256, 0, s>>>(sched, p, words, n, sched_words, err);
+        constexpr int CAP = sizeof(p) / 4;
+        return launch_dependent(patch_kernel<CAP>, (n + 255) / 256, 256, 0, s, sched, p, words, n, sched_words, err);
     });
 }
 
@@ -2506,10 +2568,9 @@ cudaError_t launch_append_tokens(int hd, const AppendTokensArgs& a0, const StepW
     return with_words(w, [&](const auto& p, const int32_t* words) {
         AppendTokensArgs a = a0;
         a.words = words;
-        if (hd == 64)
-            append_tokens_kernel<64><<<grid, kTokenThreads, 0, s>>>(a, p);
-        else
-            append_tokens_kernel<128><<<grid, kTokenThreads, 0, s>>>(a, p);
+        constexpr int CAP = sizeof(p) / 4;
+        return launch_dependent(hd == 64 ? append_tokens_kernel<64, CAP> : append_tokens_kernel<128, CAP>, grid,
+                                kTokenThreads, 0, s, a, p);
     });
 }
 
@@ -2520,10 +2581,9 @@ cudaError_t launch_rollout_step(int hd, const StepArgs& a0, const StepWords& w, 
     return with_words(w, [&](const auto& p, const int32_t* words) {
         StepArgs a = a0;
         a.words = words;
-        if (hd == 64)
-            rollout_step_kernel<64><<<grid, kStepThreads, 0, s>>>(a, p);
-        else
-            rollout_step_kernel<128><<<grid, kStepThreads, 0, s>>>(a, p);
+        constexpr int CAP = sizeof(p) / 4;
+        return launch_dependent(hd == 64 ? rollout_step_kernel<64, CAP> : rollout_step_kernel<128, CAP>, grid,
+                                kStepThreads, 0, s, a, p);
     });
 }
 
@@ -2574,10 +2634,9 @@ cudaError_t launch_gather(int hd, const GatherArgs& a, int64_t n_tokens, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t launch_decode(int hd, const DecodeArgs& a, cudaStream_t s, cudaStream_t side, cudaEvent_t fork,
-                          cudaEvent_t join) {
+cudaError_t launch_decode(int hd, const DecodeArgs& a, cudaStream_t s) {
     if (a.n_units == 0) return cudaSuccess;
-    return hd == 64 ? launch_decode_hd<64>(a, s, side, fork, join) : launch_decode_hd<128>(a, s, side, fork, join);
+    return hd == 64 ? launch_decode_hd<64>(a, s) : launch_decode_hd<128>(a, s);
 }
 
 namespace {
@@ -2586,11 +2645,7 @@ cudaError_t launch_merge_wpr(int hd, const MergeArgs& a, cudaStream_t s) {
     constexpr int kWarps = WPR > 4 ? WPR : 4;
     const int64_t warps = (int64_t)a.n * a.hq * WPR;
     const int grid = (int)std::max<int64_t>(1, (warps + kWarps - 1) / kWarps);  // one block at least: it re-arms the counters
-    if (hd == 64)
-        merge_kernel<64, WPR><<<grid, kWarps * 32, 0, s>>>(a);
-    else
-        merge_kernel<128, WPR><<<grid, kWarps * 32, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(hd == 64 ? merge_kernel<64, WPR> : merge_kernel<128, WPR>, grid, kWarps * 32, 0, s, a);
 }
 }  // namespace
 
