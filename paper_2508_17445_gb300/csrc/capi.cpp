@@ -332,8 +332,8 @@ tp_status tp_tree_create(const tp_config* cfg, tp_tree** out) {
     t->stream = (cudaStream_t)cfg->cuda_stream;
     t->pool.init(cfg->pool_blocks);
     if (cfg->pool) {
-        cudaError_t e = cudaMalloc((void**)&t->d_err, 4 * sizeof(int32_t));
-        if (e == cudaSuccess) e = cudaMemsetAsync(t->d_err, 0, 4 * sizeof(int32_t), t->stream);
+        cudaError_t e = cudaMalloc((void**)&t->d_err, 7 * sizeof(int32_t));
+        if (e == cudaSuccess) e = cudaMemsetAsync(t->d_err, 0, 7 * sizeof(int32_t), t->stream);
         if (e != cudaSuccess) {
             g_create_err = std::string("device error flag: ") + cudaGetErrorString(e);
             cudaGetLastError();
@@ -673,7 +673,7 @@ tp_status tp_prefill(tp_tree* t, const tp_node* nodes, const int32_t* n_queries,
     if (!Q || !O || !LSE || !aligned(Q, 16) || !aligned(O, 16) || !aligned(LSE, 4))
         return fail(t, TP_ERR_INVALID_ARG, "Q/O must be 16-byte and LSE 4-byte aligned device pointers");
     tp::Schedule& S = t->pf_sched;
-    tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S);
+    tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S, true);
     if (st != TP_OK) return st;
     if (S.n == 0) return TP_OK;
     // device buffer b: uploaded on the copy stream once the kernels of the
@@ -812,7 +812,7 @@ tp_status tp_debug_prefill_schedule(tp_tree* t, const tp_node* nodes, const int3
     if (!t || !len) return TP_ERR_INVALID_ARG;
     if (n < 0 || (n > 0 && (!nodes || !n_queries))) return fail(t, TP_ERR_INVALID_ARG, "bad node list");
     tp::Schedule S;
-    tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S);
+    tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S, false);
     if (st != TP_OK) return st;
     *len = (int64_t)S.words.size();
     if (cap < *len) return cap == 0 ? TP_OK : fail(t, TP_ERR_INVALID_ARG, "buffer too small");
@@ -836,7 +836,7 @@ tp_status run_schedule(tp_tree* t, const tp::Schedule& S, const void* Q, void* O
     tp::DecodeArgs a;
     if (S.prefill) {
         a.unit_pos = d_sched + S.off_unit_pos;
-        a.vis = d_sched + S.off_vis;
+        a.unit_vis = d_sched + S.off_unit_vis;
         a.out = (uint16_t*)O;
         a.out_lse = LSE;
     }
@@ -878,13 +878,12 @@ tp_status run_schedule(tp_tree* t, const tp::Schedule& S, const void* Q, void* O
     m.part_lse = a.part_lse;
     m.out = (uint16_t*)O;
     m.lse = LSE;
-    m.counters = t->d_err + 1;
     m.err = t->d_err;
     m.n_merge = S.n_merge;
     m.n_slots = S.n_slots;
-    m.n = S.n_merge > 0 ? S.n : 0;  // 0: every row was written by its only unit; only re-arm the counters
+    m.n = S.n;
     m.hq = hq;
-    {
+    if (S.n_merge > 0) {  // 0: every row was written by its only unit
         tp::LaunchTimer timer(t, tp::KK_MERGE);
         e = tp::launch_merge(hd, m, t->stream);
     }
@@ -934,7 +933,7 @@ tp_status tp_decode_noalloc(tp_tree* t, const tp_node* leaves, int32_t n, const 
     float* d_part = (float*)((uint8_t*)base + sched_bytes);
     e = cudaMemcpyAsync(d_sched, S.words.data(), S.words.size() * 4, cudaMemcpyHostToDevice, t->stream);
     if (e != cudaSuccess) return cuda_fail(t, e, "schedule upload");
-    e = cudaMemsetAsync(t->d_err + 1, 0, 3 * sizeof(int32_t), t->stream);  // unit counters start at zero
+    e = cudaMemsetAsync(t->d_err + 1, 0, 6 * sizeof(int32_t), t->stream);  // unit counters start at zero
     if (e != cudaSuccess) return cuda_fail(t, e, "counter reset");
 
     tp::DecodeArgs a;
@@ -970,7 +969,6 @@ tp_status tp_decode_noalloc(tp_tree* t, const tp_node* leaves, int32_t n, const 
     m.part_lse = a.part_lse;
     m.out = (uint16_t*)O;
     m.lse = LSE;
-    m.counters = t->d_err + 1;
     m.err = t->d_err;
     m.n_merge = S.n_merge;
     m.n_slots = S.n_slots;

@@ -110,6 +110,15 @@ constexpr int64_t kFillUnits = 152 * 2 * 6;
 constexpr int64_t kShortUnit = 8;
 constexpr int32_t kMinChunkTiles = 4;
 constexpr int32_t kMaxChunkTiles = 64;
+// Prefill row blocks: the shortest chunk worth a unit, and how many tiles the
+// longest block may have beyond an even share of the work before blocks are
+// split at all. The partials, the merge and its lists cost a call more than
+// the tail they save: split past 16 tiles against 64, a prompt of 1.1k tokens
+// took 41.5 us against 25.3, of 1.4k 48.7 / 31.2, of 1.8k 59 / 41.5; a few
+// queries on a long path are split either way (one on 30k tokens 66.6 us
+// with 1824 units as the target -> 25.0 with these).
+constexpr int64_t kPrefillMinChunk = 8;
+constexpr int64_t kPrefillMergeTiles = 64;
 
 // Stable reorder of unit records (`width` words, n_tiles in word
 // U_N_TILES) longest first (a counting sort: n_tiles <= kMaxUnitTiles).
@@ -436,7 +445,7 @@ tp_status build_schedule(tp_tree* t, const tp_node* leaves, int32_t n, uint32_t 
 }
 
 tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t* m, int32_t n, uint32_t flags,
-                                 Schedule& S) {
+                                 Schedule& S, bool device) {
     const int32_t hq = t->cfg.num_q_heads, hkv = t->cfg.num_kv_heads, g = hq / hkv;
     if (g > kTensorRowsPerUnit)
         return fail(t, TP_ERR_INVALID_ARG, "prefill needs num_q_heads / num_kv_heads <= 64");
@@ -454,50 +463,63 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     SchedScratch& X = t->scratch;
     const bool use_tc = !(flags & TP_MMA_SYNC);  // tcgen05 unless asked otherwise (measured faster)
     const int32_t occ_per_block = (use_tc ? kTcRowsPerUnit : kTensorRowsPerUnit) / g;  // whole GQA groups
-    // path tiles of every listed node, with each tile's path position
+    // path tiles of every listed node, with each tile's path position, and
+    // the tiles each row block sees (its causal clip)
     X.tiles.clear();
     X.tile_pos.clear();
+    X.block_tiles.clear();
     X.node_tile_off.assign((size_t)n + 1, 0);
-    X.vis.resize((size_t)n_q);
     int64_t work = 0;
-    for (int32_t i = 0, q0 = 0; i < n; q0 += m[i], ++i) {
+    int32_t longest = 0;
+    for (int32_t i = 0; i < n; ++i) {
         X.node_tile_off[(size_t)i] = (int32_t)X.tiles.size();
         const size_t first = X.tiles.size();
         path_tiles(t, nodes[i], X.tiles);
+        X.tile_pos.resize(X.tiles.size());
         int32_t pos = 0;
         for (size_t k = first; k < X.tiles.size(); ++k) {
-            X.tile_pos.push_back(pos);
+            X.tile_pos[k] = pos;
             pos += (X.tiles[k] & ((1 << kTileValidBits) - 1)) + 1;
         }
         const Node& nd = t->nodes[(size_t)nodes[i]];
-        const int32_t first_vis = (int32_t)(nd.path_before + nd.n_tokens - m[i]) + 1;
-        for (int32_t o = 0; o < m[i]; ++o) X.vis[(size_t)(q0 + o)] = first_vis + o;
+        const int32_t before = (int32_t)(nd.path_before + nd.n_tokens - m[i]);  // query o sees before + o + 1 tokens
+        const int32_t n_path = (int32_t)(X.tiles.size() - first);
+        const int32_t* tpos = X.tile_pos.data() + first;
+        int32_t nt = m[i] > 0 ? (int32_t)(std::lower_bound(tpos, tpos + n_path, before + 1) - tpos) : 0;
         for (int32_t o0 = 0; o0 < m[i]; o0 += occ_per_block) {
-            const int32_t o1 = std::min(m[i], o0 + occ_per_block);
-            const int32_t lim = X.vis[(size_t)(q0 + o1 - 1)];
-            const int32_t* tp0 = X.tile_pos.data() + first;
-            work += (int64_t)(std::lower_bound(tp0, tp0 + (X.tiles.size() - first), lim) - tp0) * hkv;
+            const int32_t lim = before + std::min(m[i], o0 + occ_per_block);
+            while (nt < n_path && tpos[nt] < lim) ++nt;
+            X.block_tiles.push_back(nt);
+            work += (int64_t)nt * hkv;
+            longest = std::max(longest, nt);
         }
     }
     X.node_tile_off[(size_t)n] = (int32_t)X.tiles.size();
-    const int32_t chunk = (int32_t)std::min<int64_t>(
-        kMaxUnitTiles, std::max<int64_t>(kMinChunkTiles, (work + kTargetUnits - 1) / kTargetUnits));
+    // Row blocks are cut into chunks only where the call would otherwise end
+    // on a few long ones: the longest block against an even share of the work
+    // per resident CTA, with kPrefillMergeTiles for what the partials and the
+    // merge cost.
+    const int64_t share = std::max<int64_t>(kPrefillMinChunk, (work + kResidentCtas - 1) / kResidentCtas);
+    const int32_t chunk =
+        (int32_t)std::min<int64_t>(kMaxUnitTiles, longest > share + kPrefillMergeTiles ? share : kMaxUnitTiles);
 
-    // units of 9 words while sorting: the 8 unit words and the path position
-    constexpr int W = kUnitWords + 1;
+    // units of kUnitWords + 2 words while sorting: the unit words, the path
+    // position and what the first query row sees
+    constexpr int W = kUnitWords + 2;
     std::vector<int32_t>& recs = X.units[1];
     recs.clear();
     X.pair_occ.clear();
     X.pair_slot.clear();
     int32_t n_slots = 0;
+    size_t blk = 0;
     for (int32_t i = 0, q0 = 0; i < n; q0 += m[i], ++i) {
         const int32_t toff = X.node_tile_off[(size_t)i];
-        const int32_t n_path = X.node_tile_off[(size_t)i + 1] - toff;
         const int32_t* tpos = X.tile_pos.data() + toff;
-        for (int32_t o0 = 0; o0 < m[i]; o0 += occ_per_block) {
+        const Node& nd = t->nodes[(size_t)nodes[i]];
+        const int32_t before = (int32_t)(nd.path_before + nd.n_tokens - m[i]);
+        for (int32_t o0 = 0; o0 < m[i]; o0 += occ_per_block, ++blk) {
             const int32_t o1 = std::min(m[i], o0 + occ_per_block);
-            const int32_t lim = X.vis[(size_t)(q0 + o1 - 1)];
-            const int32_t nt = (int32_t)(std::lower_bound(tpos, tpos + n_path, lim) - tpos);  // causal clip
+            const int32_t nt = X.block_tiles[blk];
             const int32_t n_chunks = (nt + chunk - 1) / chunk;
             const int32_t base = nt / n_chunks, extra = nt % n_chunks;
             for (int32_t c = 0, t0 = 0; c < n_chunks; ++c) {
@@ -507,22 +529,25 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
                     slot_base = n_slots;
                     n_slots += o1 - o0;
                     for (int32_t o = o0; o < o1; ++o)
-                        if (X.vis[(size_t)(q0 + o)] > tpos[t0]) {  // the chunk holds tokens this query sees
+                        if (before + o + 1 > tpos[t0]) {  // the chunk holds tokens this query sees
                             X.pair_occ.push_back(q0 + o);
                             X.pair_slot.push_back(slot_base + o - o0);
                         }
                 }
+                const size_t at = recs.size();
+                recs.resize(at + (size_t)hkv * W);
                 for (int32_t h = 0; h < hkv; ++h) {
                     const int32_t u[W] = {toff + t0, len, q0 + o0, 0, (o1 - o0) * g, slot_base, h,
-                                          use_tc ? KIND_TC : KIND_TENSOR, tpos[t0]};
-                    recs.insert(recs.end(), u, u + W);
+                                          use_tc ? KIND_TC : KIND_TENSOR, tpos[t0], before + o0 + 1};
+                    std::memcpy(&recs[at + (size_t)h * W], u, sizeof u);
                 }
                 t0 += len;
             }
         }
     }
     sort_units(recs, X.sorted, X.bucket, W);
-    merge_csr(X, (int32_t)n_q);
+    const bool merge = !X.pair_occ.empty();
+    if (merge || !device) merge_csr(X, (int32_t)n_q);
 
     S.prefill = true;
     S.kv_read_once = false;  // the query blocks of a path re-read its K/V
@@ -533,16 +558,22 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     S.n_occ = (int32_t)n_q;
     S.n = (int32_t)n_q;
     S.n_slots = n_slots;
-    S.n_merge = (int32_t)X.merge_slot.size();
+    S.n_merge = (int32_t)X.pair_occ.size();
+    // A unit's query rows are consecutive query tokens, so the kernels derive
+    // each row's occurrence and what it sees; the device image leaves out the
+    // lists that only say so (occurrences, visible lengths) and, without
+    // split rows, the merge lists.
+    const bool lists = !device, csr = merge || !device;
     S.off_units = kSchedHeaderWords;
     S.off_tiles = S.off_units + (int64_t)S.n_units * kUnitWords;
     S.off_occ = S.off_tiles + S.n_tiles;
-    S.off_merge_off = S.off_occ + S.n_occ;
-    S.off_merge_slot = S.off_merge_off + S.n + 1;
+    S.off_merge_off = S.off_occ + (lists ? S.n_occ : 0);
+    S.off_merge_slot = S.off_merge_off + (csr ? S.n + 1 : 0);
     S.off_unit_pos = S.off_merge_slot + S.n_merge;
     S.off_vis = S.off_unit_pos + S.n_units;
+    S.off_unit_vis = S.off_vis + (lists ? S.n : 0);
     S.off_merge_rec = 0;  // no merge records: most query rows are written directly, the rest use the CSR
-    const int64_t total = S.off_vis + S.n;
+    const int64_t total = S.off_unit_vis + (device ? S.n_units : 0);
     if (total >= (int64_t)1 << 31) return fail(t, TP_ERR_INVALID_ARG, "schedule too large");
     S.words.resize((size_t)total);
     int32_t* w = S.words.data();
@@ -559,14 +590,24 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     w[9] = S.n_tc;
     w[10] = 1;  // prefill schedule
     for (int32_t k = 0; k < S.n_units; ++k) {
-        std::memcpy(w + S.off_units + (int64_t)k * kUnitWords, &recs[(size_t)k * W], sizeof(int32_t) * kUnitWords);
-        w[S.off_unit_pos + k] = recs[(size_t)k * W + kUnitWords];
+        const int32_t* r = &recs[(size_t)k * W];
+        std::memcpy(w + S.off_units + (int64_t)k * kUnitWords, r, sizeof(int32_t) * kUnitWords);
+        w[S.off_unit_pos + k] = r[kUnitWords];
+        if (device) w[S.off_unit_vis + k] = r[kUnitWords + 1];
     }
     std::copy(X.tiles.begin(), X.tiles.end(), w + S.off_tiles);
-    for (int32_t q = 0; q < S.n; ++q) w[S.off_occ + q] = q;
-    std::copy(X.merge_off.begin(), X.merge_off.end(), w + S.off_merge_off);
-    std::copy(X.merge_slot.begin(), X.merge_slot.end(), w + S.off_merge_slot);
-    std::copy(X.vis.begin(), X.vis.end(), w + S.off_vis);
+    if (csr) {
+        std::copy(X.merge_off.begin(), X.merge_off.end(), w + S.off_merge_off);
+        std::copy(X.merge_slot.begin(), X.merge_slot.end(), w + S.off_merge_slot);
+    }
+    if (lists) {
+        for (int32_t q = 0; q < S.n; ++q) w[S.off_occ + q] = q;
+        int32_t* vis = w + S.off_vis;
+        for (int32_t i = 0; i < n; ++i) {
+            const Node& nd = t->nodes[(size_t)nodes[i]];
+            for (int32_t o = 0; o < m[i]; ++o) *vis++ = (int32_t)(nd.path_before + nd.n_tokens - m[i]) + o + 1;
+        }
+    }
     S.leaf_tail.clear();
     return TP_OK;
 }

@@ -129,11 +129,11 @@ struct DecodeArgs {
     float* part_o;      // [slot][Hq][hd], normalised partial output
     float* part_lse;    // [slot][Hq], log2-domain partial LSE
     int32_t* err;
-    const int32_t* vis = nullptr;       // prefill: visible path tokens per occurrence (nullptr: decode)
-    const int32_t* unit_pos = nullptr;  // prefill: path position of each unit's first token
+    const int32_t* unit_pos = nullptr;  // prefill: path position of each unit's first token (nullptr: decode)
+    const int32_t* unit_vis = nullptr;  // prefill: path tokens the unit's first query token sees (each next one: one more)
     uint16_t* out = nullptr;            // units with slot_base < 0 write O (bf16 [n][Hq][hd]) and
     float* out_lse = nullptr;           // LSE (natural log) here directly: their rows have no other part
-    int32_t* counters;    // [3] units claimed per kind past each CTA's first (0 at launch; the merge re-arms them)
+    int32_t* counters;    // [3] units claimed per kind, then [3] CTAs done per kind (0 at launch; the last CTA re-arms them)
     int32_t* counter;     // the counter of the launch in flight (set by the launcher)
     int32_t n_tc_units;      // units [0, n_tc) are tcgen05 units,
     int32_t n_tensor_units;  // then n_tensor mma.sync units, then CUDA-core units
@@ -160,7 +160,6 @@ struct MergeArgs {
     const float* part_lse;
     uint16_t* out;  // bf16 [n][Hq][hd]
     float* lse;     // [n][Hq], natural log
-    int32_t* counters;  // decode's three unit counters, reset to 0 here
     int32_t n;
     int32_t hq;
     int32_t* err = nullptr;  // device error word (bounds-checked build)
@@ -318,13 +317,14 @@ class BlockPool {
 struct Schedule {
     // header | units | tiles | occ | merge_off | merge_slot, then for a
     // decode schedule merge_rec [n][16], for a prefill one unit_pos
-    // [n_units] | vis [n]
+    // [n_units] | vis [n]; a prefill one for the device leaves out occ, vis
+    // and (no split rows) merge_off, and ends in unit_vis [n_units]
     std::vector<int32_t> words;
     int32_t n_units = 0, n_tiles = 0, n_occ = 0, n = 0, n_slots = 0, n_merge = 0, n_tensor = 0, n_tc = 0;
     int64_t off_units = 0, off_tiles = 0, off_occ = 0, off_merge_off = 0, off_merge_slot = 0;
     bool prefill = false;
     bool kv_read_once = false;  // see DecodeArgs::kv_read_once
-    int64_t off_unit_pos = 0, off_vis = 0, off_merge_rec = 0;
+    int64_t off_unit_pos = 0, off_vis = 0, off_unit_vis = 0, off_merge_rec = 0;
     // (leaf node, word index of the last tile of that leaf) for every place a
     // listed leaf's last block appears: appends that stay inside that block
     // change only these words (see patch_schedule)
@@ -351,7 +351,7 @@ struct SchedScratch {
     std::vector<int32_t> occ, tiles, tail_node, tail_tile;
     std::vector<int32_t> units[3], sorted, bucket;
     std::vector<int32_t> pair_occ, pair_slot, merge_off, merge_pos, merge_slot;
-    std::vector<int32_t> tile_pos, node_tile_off, vis;  // prefill
+    std::vector<int32_t> tile_pos, node_tile_off, block_tiles;  // prefill
     std::vector<int32_t> step_words;                    // words of a token step's launch
 };
 
@@ -372,7 +372,7 @@ struct tp_tree {
     tp::SchedScratch scratch;
 
     // device scratch owned by the library
-    int32_t* d_err = nullptr;  // [0] device error flag, [1..3] decode unit counters
+    int32_t* d_err = nullptr;  // [0] device error flag, [1..6] unit counters (DecodeArgs::counters)
     int32_t* d_sched = nullptr;
     int64_t d_sched_cap = 0;  // words
     float* d_part = nullptr;  // partial o then partial lse
@@ -495,8 +495,10 @@ tp_status build_schedule(tp_tree* t, const tp_node* leaves, int32_t n, uint32_t 
 // path's first vis[q] tokens; its rows are kept per node in blocks of whole
 // GQA groups, and each block reads the node's path tiles up to its last
 // visible token, in chunks of at most kMaxUnitTiles tiles.
+// device: the image the kernels read (see Schedule::words), else the whole
+// layout of tp_debug_prefill_schedule.
 tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t* m, int32_t n, uint32_t flags,
-                                 Schedule& out);
+                                 Schedule& out, bool device);
 // Refresh the last-tile words of S's leaves from the tree (valid after
 // appends that stayed inside those leaves' last blocks); `changed` receives
 // (word index, new word) pairs. Returns the number of changed words.

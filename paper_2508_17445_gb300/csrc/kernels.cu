@@ -680,6 +680,7 @@ __global__ void gather_kernel(const GatherArgs a, int64_t n_tokens) {
 struct UnitDesc {
     int tile_off, n_tiles, occ_off, row0, n_rows, slot_base, kvh, kind;
     int pos0;  // prefill: path position of the unit's first token
+    int vis0;  // and the path tokens its first query token sees
 };
 
 template <int HD>
@@ -725,7 +726,7 @@ struct Ctl {
     uint64_t qempty;          // every consumer warp holds its query fragments
     int valid[kStages][2];    // valid tokens of the stage's two tiles (0: no tile)
     int unit[2];              // published unit index (-1: no more units)
-    int desc[2][kUnitWords + 1];  // published unit descriptor (+ path position)
+    int desc[2][kUnitWords + 2];  // published unit descriptor (+ path position, first row's visible tokens)
     int tiles[2][kMaxUnitTiles];  // published unit's tile words
     int abort;
 };
@@ -1124,8 +1125,7 @@ struct TensorPath {
                     vis[h] = 0x7fffffff;
                     continue;
                 }
-                const int occ = a.occ[u.occ_off + (u.row0 + r) / a.group];
-                vis[h] = check(in_range(occ, a.ext.n), a.err) ? a.vis[occ] : 0;
+                vis[h] = u.vis0 + (u.row0 + r) / a.group;
             }
         }
 
@@ -1267,7 +1267,7 @@ struct TensorPath {
             const int qh = u.kvh * a.group + item_row % a.group;
             const float inv = 1.f / l_run[h];
             if (CAUSAL && u.slot_base < 0) {  // the row's only unit: final O and LSE
-                const int occ = a.occ[u.occ_off + item_row / a.group];
+                const int occ = u.occ_off + item_row / a.group;  // consecutive query tokens
                 if (!check(in_range(occ, a.ext.n), a.err)) continue;
                 uint16_t* dst = a.out + ((int64_t)occ * a.hq + qh) * HD;
 #pragma unroll
@@ -1293,6 +1293,17 @@ struct TensorPath {
 __device__ __forceinline__ int claim_unit(const DecodeArgs& a, int k) {
     if (a.late_wait) return a.unit_begin + atomicAdd(a.counter, 1);
     return a.unit_begin + (int)(k == 0 ? blockIdx.x : gridDim.x + atomicAdd(a.counter, 1));
+}
+
+// After a CTA's last unit: the last CTA of the launch re-arms its counters
+// (every claim was made before its CTA arrived here), so the next call, or a
+// replay of this one, needs no launch for it.
+__device__ __forceinline__ void rearm(const DecodeArgs& a) {
+    int32_t* done = a.counter + 3;
+    if (atomicAdd(done, 1) == (int)gridDim.x - 1) {
+        *a.counter = 0;
+        *done = 0;
+    }
 }
 
 // Fetcher warp: claim units, publish descriptor + tile words, stage a tensor
@@ -1341,13 +1352,17 @@ __device__ void fetch_units(const DecodeArgs& a, Ctl& c, uint8_t* qbuf) {
             dw[U_SLOT_BASE] = d.slot_base;
             dw[U_KVH] = d.kvh;
             dw[U_KIND] = d.kind;
-            dw[kUnitWords] = (u >= 0 && a.unit_pos) ? a.unit_pos[u] : 0;
+            dw[kUnitWords] = (u >= 0 && a.unit_pos) ? __ldcg(a.unit_pos + u) : 0;
+            dw[kUnitWords + 1] = (u >= 0 && a.unit_pos) ? __ldcg(a.unit_vis + u) : 0;
             *reinterpret_cast<volatile int*>(&c.unit[q]) = u;
         }
         __threadfence_block();  // every lane's tile-word stores, before lane 0 publishes
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&c.ufull[q]));  // release: slot visible to its readers
-        if (u < 0) return;
+        if (u < 0) {
+            if (lane == 0) rearm(a);
+            return;
+        }
         if constexpr (KIND == KIND_TENSOR || KIND == KIND_PREFILL) {
             // query rows of the unit: item row row0 + r is q-head
             // kvh * g + (row0 + r) % g of occurrence occ[(row0 + r) / g]
@@ -1357,7 +1372,9 @@ __device__ void fetch_units(const DecodeArgs& a, Ctl& c, uint8_t* qbuf) {
             const int g = a.group;
             for (int r = lane; r < d.n_rows; r += 32) {  // one 2*HD-byte copy per row
                 const int item_row = d.row0 + r;
-                int occ = __ldcg(a.occ + d.occ_off + item_row / g);
+                // prefill: consecutive query tokens
+                int occ = d.occ_off + item_row / g;
+                if (KIND != KIND_PREFILL) occ = __ldcg(a.occ + occ);
                 if (!check(in_range(occ, a.ext.n), a.err)) occ = 0;
                 const uint16_t* src = a.q + ((int64_t)occ * a.hq + d.kvh * g + item_row % g) * HD;
                 bulk_g2s(smem_u32(qbuf + r * Smem<HD>::kQPitch), src, HD * 2, smem_u32(&c.qfull));
@@ -1421,6 +1438,7 @@ __device__ void consume(const DecodeArgs& a, Ctl& c, uint8_t* ring, float* park,
             d.kvh = dw[U_KVH];
             d.kind = dw[U_KIND];
             d.pos0 = dw[kUnitWords];
+            d.vis0 = dw[kUnitWords + 1];
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&c.uempty[q]));
@@ -1533,7 +1551,7 @@ struct CtlTc {
     uint64_t o_free;          // the epilogue has read O (one arrival per consumer warp)
     int valid[kStages][2];
     int unit[2];
-    int desc[2][kUnitWords + 1];  // + path position of the unit's first token (prefill)
+    int desc[2][kUnitWords + 2];  // + path position, first row's visible tokens (prefill)
     int tiles[2][kMaxUnitTiles];
     uint32_t tmem;
     int abort;
@@ -1622,6 +1640,7 @@ __device__ __forceinline__ UnitDesc read_desc(const int* slot) {
     d.kvh = dw[U_KVH];
     d.kind = dw[U_KIND];
     d.pos0 = dw[kUnitWords];
+    d.vis0 = dw[kUnitWords + 1];
     return d;
 }
 
@@ -1651,7 +1670,7 @@ __device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
             const int w_slot = __shfl_sync(0xffffffffu, word, U_SLOT_BASE), w_kvh = __shfl_sync(0xffffffffu, word, U_KVH);
             const int w_kind = __shfl_sync(0xffffffffu, word, U_KIND);
             if (u >= 0 && !(w_kind == KIND_TC && unit_ok(tile_off, n_tiles, w_occ, w_row0, w_rows, w_slot, w_kvh,
-                                                         kTcRowsPerUnit, a.vis != nullptr, a.ext))) {
+                                                         kTcRowsPerUnit, a.unit_pos != nullptr, a.ext))) {
                 if (lane == 0) atomicOr(a.err, kErrBounds);  // a bad unit record: this CTA takes no more units
                 u = -1;
             }
@@ -1659,13 +1678,17 @@ __device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
         if (u >= 0)
             for (int t = lane; t < n_tiles; t += 32) c.tiles[q][t] = __ldcg(a.tiles + tile_off + t);
         if (lane < kUnitWords) reinterpret_cast<volatile int*>(c.desc[q])[lane] = word;
-        if (lane == kUnitWords)
-            reinterpret_cast<volatile int*>(c.desc[q])[lane] = (u >= 0 && a.unit_pos) ? a.unit_pos[u] : 0;
+        if (lane == kUnitWords || lane == kUnitWords + 1)
+            reinterpret_cast<volatile int*>(c.desc[q])[lane] =
+                (u >= 0 && a.unit_pos) ? __ldcg((lane == kUnitWords ? a.unit_pos : a.unit_vis) + u) : 0;
         if (lane == 0) *reinterpret_cast<volatile int*>(&c.unit[q]) = u;
         __threadfence_block();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&c.ufull[q]));
-        if (u < 0) return;
+        if (u < 0) {
+            if (lane == 0) rearm(a);
+            return;
+        }
         const int occ_off = __shfl_sync(0xffffffffu, word, U_OCC_OFF);
         const int row0 = __shfl_sync(0xffffffffu, word, U_ROW0);
         const int n_rows = __shfl_sync(0xffffffffu, word, U_N_ROWS);
@@ -1681,7 +1704,7 @@ __device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
         // async copies straight into the swizzled layout, offsets known at
         // compile time, every copy of the tile in flight at once
         constexpr int kRowsPerLane = kTcRows / 32;
-        const bool in_order = a.vis != nullptr;
+        const bool in_order = a.unit_pos != nullptr;
         int64_t src_off[kRowsPerLane];
 #pragma unroll
         for (int i = 0; i < kRowsPerLane; ++i) {
@@ -1921,10 +1944,7 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
         const int n_pairs = (d.n_tiles + 1) / 2;
         float m_used = -INFINITY, l = 0.f;
         int vis = 0x7fffffff, pos = d.pos0;
-        if (CAUSAL && row < d.n_rows) {
-            const int occ = a.occ[d.occ_off + (d.row0 + row) / a.group];
-            vis = check(in_range(occ, a.ext.n), a.err) ? a.vis[occ] : 0;
-        }
+        if (CAUSAL && row < d.n_rows) vis = d.vis0 + (d.row0 + row) / a.group;  // consecutive query tokens
         for (int j = 0; j < n_pairs; ++j) {
             const uint32_t g_stage = gs + j, sb = g_stage & 1;
             int v0 = (tw[2 * j] & ((1 << kTileValidBits) - 1)) + 1;
@@ -2061,7 +2081,7 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
             const int item_row = d.row0 + row;
             const int qh = d.kvh * a.group + item_row % a.group;
             if (final_out) {
-                const int occ = a.occ[d.occ_off + item_row / a.group];
+                const int occ = d.occ_off + item_row / a.group;
                 live = check(in_range(occ, a.ext.n), a.err);
                 dst16 = a.out + ((int64_t)occ * a.hq + qh) * HD;
                 if (live) a.out_lse[(int64_t)occ * a.hq + qh] = (m_used + __log2f(l)) * 0.69314718055994531f;
@@ -2297,7 +2317,6 @@ __global__ void __launch_bounds__(WPR > 4 ? WPR * 32 : 128) merge_kernel(const M
     const int rw =
         in_grid && a.merge_rec && lane < kMergeRecWords ? __ldcg(a.merge_rec + (int64_t)i * kMergeRecWords + lane) : -1;
     dep_wait();  // the attention kernels have completed (their schedule was there before they began)
-    if (blockIdx.x == 0 && threadIdx.x < 3) a.counters[threadIdx.x] = 0;  // re-arm their counters
     if (WPR == 1 && !in_grid) return;
     const int ns_rec = __shfl_sync(0xffffffffu, rw, 0);  // -1: the CSR (more than 15 slots, or no records)
     int ns = 0;
@@ -2444,7 +2463,7 @@ int decode_tc_grid() {
 template <int HD>
 cudaError_t launch_tc_range(DecodeArgs a, int begin, int end, int32_t* counter, cudaStream_t s) {
     if (end <= begin) return cudaSuccess;
-    const bool causal = a.vis != nullptr;
+    const bool causal = a.unit_pos != nullptr;
     const int slots = causal ? decode_tc_grid<HD, true>() : decode_tc_grid<HD, false>();
     if (slots == 0) return cudaErrorInvalidConfiguration;
     a.unit_begin = begin;
@@ -2480,7 +2499,7 @@ cudaError_t launch_decode_hd(const DecodeArgs& a, cudaStream_t s) {
     if (!tc_last) e = launch_tc_range<HD>(first, 0, tc_end, a.counters, s);
     if (e != cudaSuccess) return e;
     const DecodeArgs& m = tc_last ? first : second;
-    e = a.vis ? launch_range<HD, KIND_PREFILL>(m, tc_end, mma_end, a.counters + 1, s)
+    e = a.unit_pos ? launch_range<HD, KIND_PREFILL>(m, tc_end, mma_end, a.counters + 1, s)
               : launch_range<HD, KIND_TENSOR>(m, tc_end, mma_end, a.counters + 1, s);
     if (e == cudaSuccess && tc_last) e = launch_tc_range<HD>(second, 0, tc_end, a.counters, s);
     if (e != cudaSuccess) return e;
@@ -2644,7 +2663,7 @@ template <int WPR>
 cudaError_t launch_merge_wpr(int hd, const MergeArgs& a, cudaStream_t s) {
     constexpr int kWarps = WPR > 4 ? WPR : 4;
     const int64_t warps = (int64_t)a.n * a.hq * WPR;
-    const int grid = (int)std::max<int64_t>(1, (warps + kWarps - 1) / kWarps);  // one block at least: it re-arms the counters
+    const int grid = (int)((warps + kWarps - 1) / kWarps);
     return launch_dependent(hd == 64 ? merge_kernel<64, WPR> : merge_kernel<128, WPR>, grid, kWarps * 32, 0, s, a);
 }
 }  // namespace

@@ -1,0 +1,48 @@
+"""Where prefill row blocks are split: schedules on both sides of the rule's
+edges cover every visible token once (CPU), and the kernels, which derive each
+row's occurrence and visible length from its unit, agree with the oracle on
+split and unsplit blocks of both head sizes (GPU)."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2508_17445_gb300 as tp
+import workloads
+from test_prefill_host import check_prefill_coverage, metadata_forest
+
+# one row block (18 queries of a 7-row group at most): split past 8 + 64 tiles
+EDGES = [(72 * 32, 1), (72 * 32 + 1, 1), (73 * 32, 18), (128 * 32 + 1, 5), (40 * 32, 40), (9000, 40)]
+
+
+@pytest.mark.parametrize("flags", [0, tp.TP_MMA_SYNC])
+@pytest.mark.parametrize("tokens,queries", EDGES)
+def test_split_edges(tokens, queries, flags):
+    s = workloads.single_path(seed=1, lengths=(tokens,), heads=workloads.Heads(28, 4, 128))
+    f, ids = metadata_forest(s)
+    model = oracle.OracleForest(block_tokens=32, pool_blocks=1 << 10).replay(s)
+    check_prefill_coverage(f, model, ids, [s.leaves[0]], [queries], flags)
+    d = tp.tp_debug_prefill_schedule(f.handle, [ids[s.leaves[0]]], [queries], flags)
+    assert (d["n_slots"] > 0) == (-(-tokens // 32) > 72)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("flags", [0, tp.TP_MMA_SYNC])
+@pytest.mark.parametrize("heads", [workloads.Heads(28, 4, 128), workloads.Heads(16, 2, 64), workloads.Heads(12, 1, 128)])
+@pytest.mark.parametrize("tokens,queries", EDGES)
+def test_split_edges_against_the_oracle(tokens, queries, heads, flags):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from test_gpu_parity import _kv_source, build_forest, check
+    s = workloads.single_path(seed=2, lengths=(31, tokens - 31), heads=heads)  # the last node holds the queries
+    f, ids = build_forest(s)
+    Q = s.q("cuda:0", n=queries)
+    O, LSE = f.prefill([ids[s.leaves[0]]], [queries], Q, flags)
+    f.sync()
+    src = _kv_source(s)
+    model = oracle.OracleForest(block_tokens=32, pool_blocks=f.cfg.pool_blocks).replay(s)
+    o_ref, lse_ref = model.prefill([s.leaves[0]], [queries], Q.cpu(), src)
+    abs_src = lambda i: (src(i)[0], oracle.bf16_bits(src(i)[1]) & np.uint16(0x7FFF))  # noqa: E731
+    a_ref, _ = model.prefill([s.leaves[0]], [queries], Q.cpu(), abs_src)
+    check(O, LSE, o_ref, lse_ref, a_ref)
+    f.close()
