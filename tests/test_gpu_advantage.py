@@ -1,0 +1,48 @@
+"""The tree advantage over the sizes where its launch changes: one CTA and
+several, the last output of a CTA, one to four warps of outputs per CTA, and
+more outputs than the cooperative launch has threads (then four launches);
+paths deeper than the ancestors a thread keeps. Oracle and tolerance of
+test_gpu_rollout.py (fp64 accumulation, fp32 output: 1e-6 (|adv| + 1))."""
+import numpy as np
+import pytest
+
+from test_gpu_parity import _built  # noqa: F401
+from test_gpu_rollout import check_advantage
+
+pytestmark = pytest.mark.gpu
+
+
+def flat_trees(n_out, width, depth, seed):
+    """Prompts of `width` trajectories: a shared chain of depth // 2, then one of its own each."""
+    rng = np.random.default_rng(seed)
+    parent, leaf = [], []
+    while len(leaf) < n_out:
+        parent.append(-1)
+        top = len(parent) - 1
+        for _ in range(depth // 2):
+            parent.append(top)
+            top = len(parent) - 1
+        for _ in range(min(width, n_out - len(leaf))):
+            x = top
+            for _ in range(max(1, depth - depth // 2)):
+                parent.append(x)
+                x = len(parent) - 1
+            leaf.append(x)
+    return np.array(parent, np.int32), leaf, rng.random(n_out).round(2)
+
+
+@pytest.mark.parametrize("n_out", [1, 2, 31, 32, 33, 128, 9728, 9729, 19457, 38912, 38913])
+def test_outputs_per_launch(n_out):
+    check_advantage(*flat_trees(n_out, 16, 3, n_out))
+
+
+@pytest.mark.parametrize("depth", [1, 63, 64, 65, 66, 200])
+def test_deep_paths(depth):
+    check_advantage(*flat_trees(100, 7, depth, depth))
+
+
+def test_all_equal_and_negative_rewards():
+    parent, leaf, reward = flat_trees(64, 16, 4, 1)
+    check_advantage(parent, leaf, np.full(64, 0.25))
+    reward = np.where(np.arange(64) < 16, -3.5, reward - 0.5)  # the first prompt's are all equal
+    check_advantage(parent, leaf, reward)
