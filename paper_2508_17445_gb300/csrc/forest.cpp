@@ -97,16 +97,16 @@ void path_tiles(const tp_tree* t, tp_node leaf, std::vector<int32_t>& tiles) {
 namespace {
 constexpr int64_t kTargetUnits = 152 * 2 * 6;  // SMs x resident CTAs x waves
 constexpr int64_t kResidentCtas = 152 * 2;
-// Units a decode call is cut into where its partials allow (see the unit
-// length limit in build_schedule). Measured, whole call against no limit:
-// 16 leaves of 1.2k tokens 27.4 -> 17.3 us, 4 leaves of 8k 36.2 -> 28.0, 32
-// leaves of 2.7k 37.8 -> 30.0, 32 diverging 8k paths 73.0 -> 62.2, 64 leaves
-// over a 2k prefix (64 heads) 76.9 -> 62.8, 256 diverging paths 284 -> 261;
-// 912 units lost up to 10% of these gains and 2432 or 3648 cost calls of 64
-// independent 4k paths 3.5%. Calls of 512 leaves and more are not changed.
-constexpr int64_t kFillUnits = 152 * 2 * 6;
-// 8 blocks against 4: 32 leaves of 2.7k 30.0 against 32.9 us, 64 leaves of
-// 2.7k 43.7 against 46.9, 64 leaves of 340 tokens 12.9 against 13.9.
+// Units a decode call is cut into where its blocks allow, two for every
+// resident CTA (see the unit length limit in build_schedule). Measured, whole
+// calls without a limit against this one: 16 leaves of 1.1k tokens 22.1 ->
+// 12.0 us, four 8k paths 25.6 -> 19.8, 16 leaves of 2.7k 19.7 -> 17.9, 64
+// leaves of 1.1k 27.2 -> 20.0. With six per CTA instead: 64 leaves over a 2k
+// prefix (64 heads) 56.5 us against 50.5, 32 diverging 8k paths 53.6 / 50.7,
+// 128 leaves of 2.7k 54.3 / 52.0, 256 leaves of 1.1k 42.7 / 40.6.
+constexpr int64_t kFillUnits = kResidentCtas * 2;
+// 8 blocks against 4 (once 4-block units no longer run all at once): 32
+// leaves of 2.7k tokens 24.2 against 26.6 us, 64 leaves 35.2 / 39.7.
 constexpr int64_t kShortUnit = 8;
 constexpr int32_t kMinChunkTiles = 4;
 constexpr int32_t kMaxChunkTiles = 64;

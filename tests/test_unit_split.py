@@ -32,7 +32,7 @@ def test_units_of_calls_that_do_not_fill_the_gpu(prompt, leaf_tokens, flags):
     blocks = sum(lens.values()) * heads.num_kv_heads
     if blocks < 152 or flags & tp.TP_DECODE_NO_SHARE:  # not limited
         return
-    limit = max(4 if blocks < 4 * 304 else 8, -(-blocks // 1824))
+    limit = max(4 if blocks < 4 * 304 else 8, -(-blocks // 608))
     assert max(lens.values()) <= limit
     # only a node's own remainder is shorter than half the limit
     node_blocks = {-(-t // BT) for t in (sum(prompt), *leaf_tokens)}
@@ -45,8 +45,8 @@ def test_noalloc_takes_calls_whose_finer_schedule_does_not_fit():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     # 64 query heads: 33 KB of partials per slot, so 32 MiB hold about 1000
-    s = workloads.wide_prefix(seed=2, n_prompts=2)
-    h = s.heads
+    h = workloads.Heads(64, 1, 128)
+    s = workloads.shared_prompt(seed=2, prompt=9000, n_leaves=64, leaf_tokens=(600,) * 64, heads=h)
     f = tp.Forest(h.num_q_heads, h.num_kv_heads, h.head_dim, pool_blocks=s.upper_bound_blocks(32) + 8, device="cuda:0")
     ids = f.replay(s.ops, kv_fn=lambda i: s.kv(i, "cuda:0"))
     leaves = [ids[x] for x in s.leaves]
