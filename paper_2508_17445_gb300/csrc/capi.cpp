@@ -229,7 +229,7 @@ tp_status ensure_device(tp_tree* t, T*& ptr, int64_t& cap, int64_t need, const c
 }
 
 tp_status run_schedule(tp_tree* t, const tp::Schedule& S, const void* Q, void* O, float* LSE,
-                       const int32_t* d_sched = nullptr);
+                       const int32_t* d_sched = nullptr, const tp::StepWords* words = nullptr);
 
 // What a schedule's words index into (checked by the bounds-checked build).
 tp::Extents extents_of(const tp_tree* t, const tp::Schedule& S) {
@@ -676,6 +676,12 @@ tp_status tp_prefill(tp_tree* t, const tp_node* nodes, const int32_t* n_queries,
     tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S, true);
     if (st != TP_OK) return st;
     if (S.n == 0) return TP_OK;
+    // A small schedule without split rows travels with the attention launch:
+    // no buffer, copy stream or event (calls back to back: 40 queries 14.5 ->
+    // 9.6 us, a 717-token prompt 20.9 -> 16.8).
+    const tp::StepWords params{S.words.data(), nullptr, (int64_t)S.words.size()};
+    if (S.n_merge == 0 && S.n_tc == S.n_units && params.n <= tp::kParamWords)
+        return run_schedule(t, S, Q, O, LSE, nullptr, &params);
     // device buffer b: uploaded on the copy stream once the kernels of the
     // call two back (its last reader) are done; the attention waits for it
     cudaError_t e = cudaSuccess;
@@ -825,18 +831,27 @@ tp_status tp_debug_prefill_schedule(tp_tree* t, const tp_node* nodes, const int3
 
 namespace {
 // Launch the attention and merge kernels of a schedule already on the
-// device (at d_sched; the decode cache's t->d_sched when null).
-tp_status run_schedule(tp_tree* t, const tp::Schedule& S, const void* Q, void* O, float* LSE, const int32_t* d_sched) {
+// device (at d_sched; the decode cache's t->d_sched when null), or of one
+// whose words travel with the launch.
+tp_status run_schedule(tp_tree* t, const tp::Schedule& S, const void* Q, void* O, float* LSE, const int32_t* d_sched,
+                       const tp::StepWords* words) {
     if (!d_sched) d_sched = t->d_sched;
     const int32_t hq = t->cfg.num_q_heads, hd = t->cfg.head_dim;
     const int64_t part_floats = (int64_t)S.n_slots * hq * (hd + 1);
-    tp_status st = ensure_device(t, t->d_part, t->d_part_cap, std::max<int64_t>(part_floats, 1), "partial buffer");
-    if (st != TP_OK) return st;
+    if (part_floats > 0) {
+        tp_status st = ensure_device(t, t->d_part, t->d_part_cap, part_floats, "partial buffer");
+        if (st != TP_OK) return st;
+    }
 
     tp::DecodeArgs a;
     if (S.prefill) {
         a.unit_pos = d_sched + S.off_unit_pos;
+        a.prefill = 1;
         a.unit_vis = d_sched + S.off_unit_vis;
+        a.w_units = (int32_t)S.off_units;
+        a.w_tiles = (int32_t)S.off_tiles;
+        a.w_unit_pos = (int32_t)S.off_unit_pos;
+        a.w_unit_vis = (int32_t)S.off_unit_vis;
         a.out = (uint16_t*)O;
         a.out_lse = LSE;
     }
@@ -865,7 +880,7 @@ tp_status run_schedule(tp_tree* t, const tp::Schedule& S, const void* Q, void* O
     cudaError_t e = cudaSuccess;
     if (a.n_units > 0) {
         tp::LaunchTimer timer(t, tp::KK_DECODE);
-        e = tp::launch_decode(hd, a, t->stream);
+        e = tp::launch_decode(hd, a, t->stream, words);
         timer.kernels((S.n_tc > 0) + (S.n_tensor > 0) + (S.n_units > S.n_tc + S.n_tensor));
     }
     if (e != cudaSuccess) return cuda_fail(t, e, "decode kernel");

@@ -129,8 +129,11 @@ struct DecodeArgs {
     float* part_o;      // [slot][Hq][hd], normalised partial output
     float* part_lse;    // [slot][Hq], log2-domain partial LSE
     int32_t* err;
-    const int32_t* unit_pos = nullptr;  // prefill: path position of each unit's first token (nullptr: decode)
+    int32_t prefill = 0;
+    const int32_t* unit_pos = nullptr;  // prefill: path position of each unit's first token
     const int32_t* unit_vis = nullptr;  // prefill: path tokens the unit's first query token sees (each next one: one more)
+    // a schedule that travels with the launch (StepWords): its sections' first words
+    int32_t w_units = 0, w_tiles = 0, w_unit_pos = 0, w_unit_vis = 0;
     uint16_t* out = nullptr;            // units with slot_base < 0 write O (bf16 [n][Hq][hd]) and
     float* out_lse = nullptr;           // LSE (natural log) here directly: their rows have no other part
     int32_t* counters;    // [3] units claimed per kind, then [3] CTAs done per kind (0 at launch; the last CTA re-arms them)
@@ -273,7 +276,9 @@ int64_t advantage_ws_bytes(int64_t n_nodes, int64_t n_out);
 
 // Launchers (kernels.cu). Return cudaSuccess or the launch error.
 cudaError_t launch_append(int head_dim, const AppendArgs& a, cudaStream_t s);
-cudaError_t launch_decode(int head_dim, const DecodeArgs& a, cudaStream_t s);
+// words: the schedule's words when they travel with the launch (tcgen05 units
+// only, at most kParamWords), else null.
+cudaError_t launch_decode(int head_dim, const DecodeArgs& a, cudaStream_t s, const StepWords* words = nullptr);
 cudaError_t launch_merge(int head_dim, const MergeArgs& a, cudaStream_t s);
 cudaError_t launch_gather(int head_dim, const GatherArgs& a, int64_t n_tokens, cudaStream_t s);
 // sched[pairs[2k]] = pairs[2k + 1] for k < n (sched_words and err: the

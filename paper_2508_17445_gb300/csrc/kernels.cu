@@ -1499,8 +1499,8 @@ __device__ void fetch_units(const DecodeArgs& a, Ctl& c, uint8_t* qbuf) {
             dw[U_SLOT_BASE] = d.slot_base;
             dw[U_KVH] = d.kvh;
             dw[U_KIND] = d.kind;
-            dw[kUnitWords] = (u >= 0 && a.unit_pos) ? __ldcg(a.unit_pos + u) : 0;
-            dw[kUnitWords + 1] = (u >= 0 && a.unit_pos) ? __ldcg(a.unit_vis + u) : 0;
+            dw[kUnitWords] = (u >= 0 && a.prefill) ? __ldcg(a.unit_pos + u) : 0;
+            dw[kUnitWords + 1] = (u >= 0 && a.prefill) ? __ldcg(a.unit_vis + u) : 0;
             *reinterpret_cast<volatile int*>(&c.unit[q]) = u;
         }
         __threadfence_block();  // every lane's tile-word stores, before lane 0 publishes
@@ -1795,8 +1795,12 @@ __device__ __forceinline__ UnitDesc read_desc(const int* slot) {
 // in the 128-byte-swizzle K-major layout the MMA reads. Rows past n_rows are
 // left as they are: a row of A only reaches the same row of S, P and O, and
 // those rows are never written out.
-template <int HD>
-__device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
+template <int HD, int CAP>
+__device__ void tc_fetch(const DecodeArgs& a, const ParamWords<CAP>& p, CtlTc& c, uint8_t* qbuf) {
+    // schedule words: on the device, or in the launch's parameter (prefill)
+    auto word_at = [&](const int32_t* section, int32_t first, int64_t i) {
+        return CAP == 1 ? __ldcg(section + i) : p.v[first + i];
+    };
     const int lane = threadIdx.x & 31;
     volatile int* abort = &c.abort;
     for (int k = 0;; ++k) {
@@ -1808,7 +1812,7 @@ __device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
             if (u >= a.unit_end) u = -1;
         }
         u = __shfl_sync(0xffffffffu, u, 0);
-        const int word = (u >= 0 && lane < kUnitWords) ? __ldcg(a.units + (int64_t)u * kUnitWords + lane) : 0;
+        const int word = (u >= 0 && lane < kUnitWords) ? word_at(a.units, a.w_units, (int64_t)u * kUnitWords + lane) : 0;
         const int n_tiles = __shfl_sync(0xffffffffu, word, U_N_TILES);
         const int tile_off = __shfl_sync(0xffffffffu, word, U_TILE_OFF);
         if constexpr (kBoundsCheck) {
@@ -1817,17 +1821,19 @@ __device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
             const int w_slot = __shfl_sync(0xffffffffu, word, U_SLOT_BASE), w_kvh = __shfl_sync(0xffffffffu, word, U_KVH);
             const int w_kind = __shfl_sync(0xffffffffu, word, U_KIND);
             if (u >= 0 && !(w_kind == KIND_TC && unit_ok(tile_off, n_tiles, w_occ, w_row0, w_rows, w_slot, w_kvh,
-                                                         kTcRowsPerUnit, a.unit_pos != nullptr, a.ext))) {
+                                                         kTcRowsPerUnit, a.prefill != 0, a.ext))) {
                 if (lane == 0) atomicOr(a.err, kErrBounds);  // a bad unit record: this CTA takes no more units
                 u = -1;
             }
         }
         if (u >= 0)
-            for (int t = lane; t < n_tiles; t += 32) c.tiles[q][t] = __ldcg(a.tiles + tile_off + t);
+            for (int t = lane; t < n_tiles; t += 32) c.tiles[q][t] = word_at(a.tiles, a.w_tiles, tile_off + t);
         if (lane < kUnitWords) reinterpret_cast<volatile int*>(c.desc[q])[lane] = word;
         if (lane == kUnitWords || lane == kUnitWords + 1)
             reinterpret_cast<volatile int*>(c.desc[q])[lane] =
-                (u >= 0 && a.unit_pos) ? __ldcg((lane == kUnitWords ? a.unit_pos : a.unit_vis) + u) : 0;
+                u < 0 || !a.prefill      ? 0
+                : lane == kUnitWords ? word_at(a.unit_pos, a.w_unit_pos, u)
+                                     : word_at(a.unit_vis, a.w_unit_vis, u);
         if (lane == 0) *reinterpret_cast<volatile int*>(&c.unit[q]) = u;
         __threadfence_block();
         __syncwarp();
@@ -1851,13 +1857,13 @@ __device__ void tc_fetch(const DecodeArgs& a, CtlTc& c, uint8_t* qbuf) {
         // async copies straight into the swizzled layout, offsets known at
         // compile time, every copy of the tile in flight at once
         constexpr int kRowsPerLane = kTcRows / 32;
-        const bool in_order = a.unit_pos != nullptr;
+        const bool in_order = a.prefill != 0;
         int64_t src_off[kRowsPerLane];
 #pragma unroll
         for (int i = 0; i < kRowsPerLane; ++i) {
             const int r = lane + 32 * i;
-            const int item_row = row0 + r, p = item_row / g, hh = item_row - p * g;
-            int occ = r >= n_rows ? 0 : in_order ? occ_off + p : __ldcg(a.occ + occ_off + p);
+            const int item_row = row0 + r, po = item_row / g, hh = item_row - po * g;
+            int occ = r >= n_rows ? 0 : in_order ? occ_off + po : __ldcg(a.occ + occ_off + po);
             if (!check(in_range(occ, a.ext.n), a.err)) occ = 0;
             src_off[i] = ((int64_t)occ * a.hq + kvh * g + hh) * HD;
         }
@@ -2287,8 +2293,9 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
     }
 }
 
-template <int HD, bool CAUSAL>
-__global__ void __launch_bounds__(kTcThreads, 2) decode_tc_kernel(const DecodeArgs a) {
+template <int HD, bool CAUSAL, int CAP>
+__global__ void __launch_bounds__(kTcThreads, 2)
+    decode_tc_kernel(const DecodeArgs a, const __grid_constant__ ParamWords<CAP> words) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(16) CtlTc ctl;
     // 128-byte-swizzle operands need 1024-byte-aligned atoms
@@ -2335,7 +2342,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) decode_tc_kernel(const DecodeAr
     else if (warp == kTcStreamerWarp) {
         if ((tid & 31) == 0) tc_stream<HD>(a, ctl, ring);
     } else if (warp == kTcFetcherWarp) {
-        tc_fetch<HD>(a, ctl, qbuf);
+        tc_fetch<HD, CAP>(a, words, ctl, qbuf);
     } else if (warp == kTcIssuerWarp) {
         if ((tid & 31) == 0) tc_issue<HD>(a, ctl, ring, qbuf);
     }
@@ -2529,6 +2536,23 @@ __global__ void __launch_bounds__(WPR > 4 ? WPR * 32 : 128) merge_kernel(const M
     if (lane == 0) a.lse[(int64_t)i * a.hq + qh] = (M + __log2f(L)) * 0.69314718055994531f;
 }
 
+// Calls launch(ParamWords, device words) with the words in the smallest
+// parameter that holds them: 2 KB, 16 KB, or the device copy.
+template <typename Launch>
+cudaError_t with_words(const StepWords& w, Launch launch) {
+    if (w.n <= kParamWordsSmall) {
+        ParamWords<kParamWordsSmall> p;
+        std::copy(w.host, w.host + w.n, p.v);
+        return launch(p, (const int32_t*)nullptr);
+    }
+    if (w.n <= kParamWords) {
+        ParamWords<kParamWords> p;
+        std::copy(w.host, w.host + w.n, p.v);
+        return launch(p, (const int32_t*)nullptr);
+    }
+    return launch(ParamWords<1>{}, w.device);
+}
+
 // Launch that may start while its predecessor on the stream still runs (the
 // kernel waits for it with dep_wait).
 template <typename... P, typename... A>
@@ -2576,16 +2600,16 @@ cudaError_t launch_range(DecodeArgs a, int begin, int end, int32_t* counter, cud
                             decode_smem<HD, KIND>(), s, a);
 }
 
-template <int HD, bool CAUSAL>
+template <int HD, bool CAUSAL, int CAP>
 int decode_tc_grid() {
     static int grid = [] {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaFuncSetAttribute(decode_tc_kernel<HD, CAUSAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(decode_tc_kernel<HD, CAUSAL, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  TcSmem<HD>::kBytes) != cudaSuccess)
             return 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_tc_kernel<HD, CAUSAL>, kTcThreads,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_tc_kernel<HD, CAUSAL, CAP>, kTcThreads,
                                                           TcSmem<HD>::kBytes) != cudaSuccess)
             return 0;
         // The occupancy query answers 1 for this kernel on GB300 although its
@@ -2595,7 +2619,7 @@ int decode_tc_grid() {
         // unit counter exhausted and exits.
         cudaFuncAttributes fa{};
         int smem_sm = 0, reserved = 0;
-        if (cudaFuncGetAttributes(&fa, decode_tc_kernel<HD, CAUSAL>) != cudaSuccess) return 0;
+        if (cudaFuncGetAttributes(&fa, decode_tc_kernel<HD, CAUSAL, CAP>) != cudaSuccess) return 0;
         cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
         const int by_smem = smem_sm / (int)(TcSmem<HD>::kBytes + fa.sharedSizeBytes + reserved);
@@ -2607,17 +2631,27 @@ int decode_tc_grid() {
     return grid;
 }
 
-template <int HD>
-cudaError_t launch_tc_range(DecodeArgs a, int begin, int end, int32_t* counter, cudaStream_t s) {
-    if (end <= begin) return cudaSuccess;
-    const bool causal = a.unit_pos != nullptr;
-    const int slots = causal ? decode_tc_grid<HD, true>() : decode_tc_grid<HD, false>();
+template <int HD, bool CAUSAL, int CAP>
+cudaError_t launch_tc_kernel(const DecodeArgs& a, int n_units, cudaStream_t s, const ParamWords<CAP>& words) {
+    const int slots = decode_tc_grid<HD, CAUSAL, CAP>();
     if (slots == 0) return cudaErrorInvalidConfiguration;
+    return launch_dependent(decode_tc_kernel<HD, CAUSAL, CAP>, std::min(n_units, slots), kTcThreads, TcSmem<HD>::kBytes,
+                            s, a, words);
+}
+
+template <int HD>
+cudaError_t launch_tc_range(DecodeArgs a, int begin, int end, int32_t* counter, cudaStream_t s,
+                            const StepWords* words = nullptr) {
+    if (end <= begin) return cudaSuccess;
     a.unit_begin = begin;
     a.unit_end = end;
     a.counter = counter;
-    return launch_dependent(causal ? decode_tc_kernel<HD, true> : decode_tc_kernel<HD, false>,
-                            std::min(end - begin, slots), kTcThreads, TcSmem<HD>::kBytes, s, a);
+    if (words)  // prefill
+        return with_words(*words, [&](const auto& p, const int32_t*) {
+            return launch_tc_kernel<HD, true>(a, end - begin, s, p);
+        });
+    return a.prefill ? launch_tc_kernel<HD, true>(a, end - begin, s, ParamWords<1>{})
+                     : launch_tc_kernel<HD, false>(a, end - begin, s, ParamWords<1>{});
 }
 
 // Both attention kernels of a call run side by side: the second is launched
@@ -2637,16 +2671,16 @@ cudaError_t launch_tc_range(DecodeArgs a, int begin, int end, int32_t* counter, 
 constexpr int kTcLastUnits = 11 * 152;
 
 template <int HD>
-cudaError_t launch_decode_hd(const DecodeArgs& a, cudaStream_t s) {
+cudaError_t launch_decode_hd(const DecodeArgs& a, cudaStream_t s, const StepWords* words) {
     const int tc_end = a.n_tc_units, mma_end = tc_end + a.n_tensor_units;
     const bool tc_last = tc_end >= kTcLastUnits && mma_end > tc_end;
     DecodeArgs first = a, second = a;
     second.late_wait = tc_end > 0 && mma_end > tc_end;
     cudaError_t e = cudaSuccess;
-    if (!tc_last) e = launch_tc_range<HD>(first, 0, tc_end, a.counters, s);
+    if (!tc_last) e = launch_tc_range<HD>(first, 0, tc_end, a.counters, s, words);
     if (e != cudaSuccess) return e;
     const DecodeArgs& m = tc_last ? first : second;
-    e = a.unit_pos ? launch_range<HD, KIND_PREFILL>(m, tc_end, mma_end, a.counters + 1, s)
+    e = a.prefill ? launch_range<HD, KIND_PREFILL>(m, tc_end, mma_end, a.counters + 1, s)
               : launch_range<HD, KIND_TENSOR>(m, tc_end, mma_end, a.counters + 1, s);
     if (e == cudaSuccess && tc_last) e = launch_tc_range<HD>(second, 0, tc_end, a.counters, s);
     if (e != cudaSuccess) return e;
@@ -2701,25 +2735,6 @@ cudaError_t launch_wait_probe(int32_t* err, uint64_t limit_ns, cudaStream_t s) {
     wait_probe_kernel<<<1, 32, 0, s>>>(err, limit_ns);
     return cudaGetLastError();
 }
-
-// Calls launch(ParamWords, device words) with the words in the smallest
-// parameter that holds them: 2 KB, 16 KB, or the device copy.
-namespace {
-template <typename Launch>
-cudaError_t with_words(const StepWords& w, Launch launch) {
-    if (w.n <= kParamWordsSmall) {
-        ParamWords<kParamWordsSmall> p;
-        std::copy(w.host, w.host + w.n, p.v);
-        return launch(p, (const int32_t*)nullptr);
-    }
-    if (w.n <= kParamWords) {
-        ParamWords<kParamWords> p;
-        std::copy(w.host, w.host + w.n, p.v);
-        return launch(p, (const int32_t*)nullptr);
-    }
-    return launch(ParamWords<1>{}, w.device);
-}
-}  // namespace
 
 cudaError_t launch_patch(int32_t* sched, const StepWords& pairs, int32_t n, cudaStream_t s, int64_t sched_words,
                          int32_t* err) {
@@ -2815,9 +2830,9 @@ cudaError_t launch_gather(int hd, const GatherArgs& a, int64_t n_tokens, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t launch_decode(int hd, const DecodeArgs& a, cudaStream_t s) {
+cudaError_t launch_decode(int hd, const DecodeArgs& a, cudaStream_t s, const StepWords* words) {
     if (a.n_units == 0) return cudaSuccess;
-    return hd == 64 ? launch_decode_hd<64>(a, s) : launch_decode_hd<128>(a, s);
+    return hd == 64 ? launch_decode_hd<64>(a, s, words) : launch_decode_hd<128>(a, s, words);
 }
 
 namespace {

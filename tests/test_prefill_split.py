@@ -46,3 +46,32 @@ def test_split_edges_against_the_oracle(tokens, queries, heads, flags):
     a_ref, _ = model.prefill([s.leaves[0]], [queries], Q.cpu(), abs_src)
     check(O, LSE, o_ref, lse_ref, a_ref)
     f.close()
+
+
+# schedules of a little under and over 512 and 4096 words (4 units of 10 words per 18 queries): two parameter sizes of
+# the launch, then an upload; calls back to back, each with a schedule of its own
+@pytest.mark.gpu
+def test_schedule_words_with_the_launch():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from test_gpu_parity import _kv_source, build_forest, check
+    heads = workloads.Heads(28, 4, 128)
+    sizes = [18, 198, 216, 217, 1782, 1800, 1818, 1900, 1, 217]
+    cases = []
+    for i, n in enumerate(sizes):
+        s = workloads.single_path(seed=20 + i, lengths=(n,), heads=heads)
+        f, ids = build_forest(s)
+        cases.append((s, f, ids[s.leaves[0]], n, s.q("cuda:0", n=n)))
+    torch.cuda.synchronize()
+    words = [len(tp.tp_debug_prefill_schedule(f.handle, [x], [n])["units"]) * 10 + 16 for _, f, x, n, _ in cases]
+    assert min(words) < 512 < words[3] < 4096 < max(words)
+    outs = [f.prefill([x], [n], Q) for _, f, x, n, Q in cases]
+    torch.cuda.synchronize()
+    for (s, f, x, n, Q), (O, LSE) in zip(cases, outs):
+        f.sync()
+        rows = sorted({0, n // 2, n - 1} | set(range(0, n, 97)))
+        model = oracle.OracleForest(block_tokens=32, pool_blocks=f.cfg.pool_blocks).replay(s)
+        o_ref, lse_ref = model.prefill([s.leaves[0]], [n], Q.cpu(), _kv_source(s), indices=rows)
+        check(O, LSE, o_ref, lse_ref, rows=rows)
+        f.close()
