@@ -120,10 +120,10 @@ constexpr int32_t kMaxChunkTiles = 64;
 constexpr int64_t kPrefillMinChunk = 8;
 constexpr int64_t kPrefillMergeTiles = 64;
 
-// Stable reorder of unit records (`width` words, n_tiles in word
-// U_N_TILES) longest first (a counting sort: n_tiles <= kMaxUnitTiles).
-void sort_units(std::vector<int32_t>& u, std::vector<int32_t>& out, std::vector<int32_t>& bucket,
-                size_t width = kUnitWords) {
+// Stable reorder of unit records longest first (a counting sort: n_tiles <=
+// kMaxUnitTiles).
+void sort_units(std::vector<int32_t>& u, std::vector<int32_t>& out, std::vector<int32_t>& bucket) {
+    constexpr size_t width = kUnitWords;
     const size_t cnt = u.size() / width;
     if (cnt < 2) return;
     bucket.assign(kMaxUnitTiles + 2, 0);
@@ -463,8 +463,9 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     SchedScratch& X = t->scratch;
     const bool use_tc = !(flags & TP_MMA_SYNC);  // tcgen05 unless asked otherwise (measured faster)
     const int32_t occ_per_block = (use_tc ? kTcRowsPerUnit : kTensorRowsPerUnit) / g;  // whole GQA groups
-    // path tiles of every listed node, with each tile's path position, and
-    // the tiles each row block sees (its causal clip)
+    // 1. path tiles of every listed node, with each tile's path position (a
+    //    sibling of the node before copies what lies above them both), and
+    //    the tiles each row block sees (its causal clip)
     X.tiles.clear();
     X.tile_pos.clear();
     X.block_tiles.clear();
@@ -472,16 +473,29 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     int64_t work = 0;
     int32_t longest = 0;
     for (int32_t i = 0; i < n; ++i) {
-        X.node_tile_off[(size_t)i] = (int32_t)X.tiles.size();
+        const Node& nd = t->nodes[(size_t)nodes[i]];
         const size_t first = X.tiles.size();
-        path_tiles(t, nodes[i], X.tiles);
-        X.tile_pos.resize(X.tiles.size());
+        X.node_tile_off[(size_t)i] = (int32_t)first;
         int32_t pos = 0;
-        for (size_t k = first; k < X.tiles.size(); ++k) {
+        size_t at = first;  // tiles from here on have no position yet
+        if (i > 0 && nd.parent != -1 && nd.parent == t->nodes[(size_t)nodes[i - 1]].parent) {
+            const size_t prev = (size_t)X.node_tile_off[(size_t)i - 1];
+            const size_t above = first - prev - t->nodes[(size_t)nodes[i - 1]].blocks.size();
+            X.tiles.resize(first + above);
+            X.tile_pos.resize(first + above);
+            std::copy_n(X.tiles.data() + prev, above, X.tiles.data() + first);
+            std::copy_n(X.tile_pos.data() + prev, above, X.tile_pos.data() + first);
+            at += above;
+            pos = (int32_t)nd.path_before;
+            node_tiles(t, nd, X.tiles);
+        } else {
+            path_tiles(t, nodes[i], X.tiles);
+        }
+        X.tile_pos.resize(X.tiles.size());
+        for (size_t k = at; k < X.tiles.size(); ++k) {
             X.tile_pos[k] = pos;
             pos += (X.tiles[k] & ((1 << kTileValidBits) - 1)) + 1;
         }
-        const Node& nd = t->nodes[(size_t)nodes[i]];
         const int32_t before = (int32_t)(nd.path_before + nd.n_tokens - m[i]);  // query o sees before + o + 1 tokens
         const int32_t n_path = (int32_t)(X.tiles.size() - first);
         const int32_t* tpos = X.tile_pos.data() + first;
@@ -495,23 +509,63 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
         }
     }
     X.node_tile_off[(size_t)n] = (int32_t)X.tiles.size();
-    // Row blocks are cut into chunks only where the call would otherwise end
-    // on a few long ones: the longest block against an even share of the work
-    // per resident CTA, with kPrefillMergeTiles for what the partials and the
-    // merge cost.
+    // 2. Row blocks are cut into chunks only where the call would otherwise
+    //    end on a few long ones: the longest block against an even share of
+    //    the work per resident CTA, with kPrefillMergeTiles for what the
+    //    partials and the merge cost.
     const int64_t share = std::max<int64_t>(kPrefillMinChunk, (work + kResidentCtas - 1) / kResidentCtas);
     const int32_t chunk =
         (int32_t)std::min<int64_t>(kMaxUnitTiles, longest > share + kPrefillMergeTiles ? share : kMaxUnitTiles);
+    // 3. units longest first (stable): their number per length, then each
+    //    block's units straight to their places in the schedule (with records
+    //    built, sorted and split, ragged calls waited for the host: 2160 units
+    //    70 us a call against 56, now the GPU's time)
+    X.bucket.assign(kMaxUnitTiles + 2, 0);
+    int32_t n_slots = 0;
+    bool merge = false;
+    size_t blk = 0;
+    for (int32_t i = 0; i < n; ++i)
+        for (int32_t o0 = 0; o0 < m[i]; o0 += occ_per_block, ++blk) {
+            const int32_t nt = X.block_tiles[blk], n_chunks = (nt + chunk - 1) / chunk;
+            const int32_t base = nt / n_chunks, extra = nt % n_chunks;
+            X.bucket[(size_t)(kMaxUnitTiles - base + 1)] += (n_chunks - extra) * hkv;
+            if (extra) X.bucket[(size_t)(kMaxUnitTiles - base)] += extra * hkv;
+            merge |= n_chunks > 1;
+        }
+    for (int b = 1; b < kMaxUnitTiles + 2; ++b) X.bucket[(size_t)b] += X.bucket[(size_t)b - 1];
 
-    // units of kUnitWords + 2 words while sorting: the unit words, the path
-    // position and what the first query row sees
-    constexpr int W = kUnitWords + 2;
-    std::vector<int32_t>& recs = X.units[1];
-    recs.clear();
+    S.prefill = true;
+    S.kv_read_once = false;  // the query blocks of a path re-read its K/V
+    S.n_units = X.bucket.back();
+    S.n_tc = use_tc ? S.n_units : 0;
+    S.n_tensor = use_tc ? 0 : S.n_units;
+    S.n_tiles = (int32_t)X.tiles.size();
+    S.n_occ = (int32_t)n_q;
+    S.n = (int32_t)n_q;
+    // A unit's query rows are consecutive query tokens, so the kernels derive
+    // each row's occurrence and what it sees; the device image leaves out the
+    // lists that only say so (occurrences, visible lengths) and, without
+    // split rows, the merge lists.
+    const bool lists = !device, csr = merge || !device;
+    S.off_units = kSchedHeaderWords;
+    S.off_tiles = S.off_units + (int64_t)S.n_units * kUnitWords;
+    auto sections = [&](int64_t n_merge) {
+        S.off_occ = S.off_tiles + S.n_tiles;
+        S.off_merge_off = S.off_occ + (lists ? S.n_occ : 0);
+        S.off_merge_slot = S.off_merge_off + (csr ? S.n + 1 : 0);
+        S.off_unit_pos = S.off_merge_slot + n_merge;
+        S.off_vis = S.off_unit_pos + S.n_units;
+        S.off_unit_vis = S.off_vis + (lists ? S.n : 0);
+        return S.off_unit_vis + (device ? S.n_units : 0);
+    };
     X.pair_occ.clear();
     X.pair_slot.clear();
-    int32_t n_slots = 0;
-    size_t blk = 0;
+    X.unit_pos.resize((size_t)S.n_units);
+    X.unit_vis.resize((size_t)S.n_units);
+    if (sections(0) >= (int64_t)1 << 31) return fail(t, TP_ERR_INVALID_ARG, "schedule too large");
+    S.words.resize((size_t)S.off_tiles);  // the rest once the number of merge entries is known
+    int32_t* units = S.words.data() + S.off_units;
+    blk = 0;
     for (int32_t i = 0, q0 = 0; i < n; q0 += m[i], ++i) {
         const int32_t toff = X.node_tile_off[(size_t)i];
         const int32_t* tpos = X.tile_pos.data() + toff;
@@ -534,46 +588,29 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
                             X.pair_slot.push_back(slot_base + o - o0);
                         }
                 }
-                const size_t at = recs.size();
-                recs.resize(at + (size_t)hkv * W);
-                for (int32_t h = 0; h < hkv; ++h) {
-                    const int32_t u[W] = {toff + t0, len, q0 + o0, 0, (o1 - o0) * g, slot_base, h,
-                                          use_tc ? KIND_TC : KIND_TENSOR, tpos[t0], before + o0 + 1};
-                    std::memcpy(&recs[at + (size_t)h * W], u, sizeof u);
+                int32_t& next = X.bucket[(size_t)(kMaxUnitTiles - len)];
+                for (int32_t h = 0; h < hkv; ++h, ++next) {
+                    int32_t* u = units + (int64_t)next * kUnitWords;
+                    u[U_TILE_OFF] = toff + t0;
+                    u[U_N_TILES] = len;
+                    u[U_OCC_OFF] = q0 + o0;
+                    u[U_ROW0] = 0;
+                    u[U_N_ROWS] = (o1 - o0) * g;
+                    u[U_SLOT_BASE] = slot_base;
+                    u[U_KVH] = h;
+                    u[U_KIND] = use_tc ? KIND_TC : KIND_TENSOR;
+                    X.unit_pos[(size_t)next] = tpos[t0];
+                    X.unit_vis[(size_t)next] = before + o0 + 1;  // what the first query row sees
                 }
                 t0 += len;
             }
         }
     }
-    sort_units(recs, X.sorted, X.bucket, W);
-    const bool merge = !X.pair_occ.empty();
-    if (merge || !device) merge_csr(X, (int32_t)n_q);
-
-    S.prefill = true;
-    S.kv_read_once = false;  // the query blocks of a path re-read its K/V
-    S.n_units = (int32_t)(recs.size() / W);
-    S.n_tc = use_tc ? S.n_units : 0;
-    S.n_tensor = use_tc ? 0 : S.n_units;
-    S.n_tiles = (int32_t)X.tiles.size();
-    S.n_occ = (int32_t)n_q;
-    S.n = (int32_t)n_q;
+    if (csr) merge_csr(X, (int32_t)n_q);
     S.n_slots = n_slots;
     S.n_merge = (int32_t)X.pair_occ.size();
-    // A unit's query rows are consecutive query tokens, so the kernels derive
-    // each row's occurrence and what it sees; the device image leaves out the
-    // lists that only say so (occurrences, visible lengths) and, without
-    // split rows, the merge lists.
-    const bool lists = !device, csr = merge || !device;
-    S.off_units = kSchedHeaderWords;
-    S.off_tiles = S.off_units + (int64_t)S.n_units * kUnitWords;
-    S.off_occ = S.off_tiles + S.n_tiles;
-    S.off_merge_off = S.off_occ + (lists ? S.n_occ : 0);
-    S.off_merge_slot = S.off_merge_off + (csr ? S.n + 1 : 0);
-    S.off_unit_pos = S.off_merge_slot + S.n_merge;
-    S.off_vis = S.off_unit_pos + S.n_units;
-    S.off_unit_vis = S.off_vis + (lists ? S.n : 0);
     S.off_merge_rec = 0;  // no merge records: most query rows are written directly, the rest use the CSR
-    const int64_t total = S.off_unit_vis + (device ? S.n_units : 0);
+    const int64_t total = sections(S.n_merge);
     if (total >= (int64_t)1 << 31) return fail(t, TP_ERR_INVALID_ARG, "schedule too large");
     S.words.resize((size_t)total);
     int32_t* w = S.words.data();
@@ -589,13 +626,9 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     w[8] = S.n_tensor;
     w[9] = S.n_tc;
     w[10] = 1;  // prefill schedule
-    for (int32_t k = 0; k < S.n_units; ++k) {
-        const int32_t* r = &recs[(size_t)k * W];
-        std::memcpy(w + S.off_units + (int64_t)k * kUnitWords, r, sizeof(int32_t) * kUnitWords);
-        w[S.off_unit_pos + k] = r[kUnitWords];
-        if (device) w[S.off_unit_vis + k] = r[kUnitWords + 1];
-    }
     std::copy(X.tiles.begin(), X.tiles.end(), w + S.off_tiles);
+    std::copy(X.unit_pos.begin(), X.unit_pos.end(), w + S.off_unit_pos);
+    if (device) std::copy(X.unit_vis.begin(), X.unit_vis.end(), w + S.off_unit_vis);
     if (csr) {
         std::copy(X.merge_off.begin(), X.merge_off.end(), w + S.off_merge_off);
         std::copy(X.merge_slot.begin(), X.merge_slot.end(), w + S.off_merge_slot);

@@ -356,7 +356,7 @@ struct SchedScratch {
     std::vector<int32_t> occ, tiles, tail_node, tail_tile;
     std::vector<int32_t> units[3], sorted, bucket;
     std::vector<int32_t> pair_occ, pair_slot, merge_off, merge_pos, merge_slot;
-    std::vector<int32_t> tile_pos, node_tile_off, block_tiles;  // prefill
+    std::vector<int32_t> tile_pos, node_tile_off, block_tiles, unit_pos, unit_vis;  // prefill
     std::vector<int32_t> step_words;                    // words of a token step's launch
 };
 
