@@ -1826,8 +1826,33 @@ __device__ void tc_fetch(const DecodeArgs& a, const ParamWords<CAP>& p, CtlTc& c
                 u = -1;
             }
         }
-        if (u >= 0)
+        const int occ_off = __shfl_sync(0xffffffffu, word, U_OCC_OFF);
+        const int row0 = __shfl_sync(0xffffffffu, word, U_ROW0);
+        const int n_rows = __shfl_sync(0xffffffffu, word, U_N_ROWS);
+        const int kvh = __shfl_sync(0xffffffffu, word, U_KVH);
+        // the source row of query rows lane, lane + 32, ... (row of Q as
+        // [n * hq]): prefill schedules list query rows in order (occurrence =
+        // query index), decode looks the occurrence up, together with the
+        // tile words
+        constexpr int kRowsPerLane = kTcRows / 32;
+        const int g = a.group;
+        uint32_t src_row[kRowsPerLane];
+        if (u >= 0) {
+            int hh[kRowsPerLane], occ[kRowsPerLane];
+#pragma unroll
+            for (int i = 0; i < kRowsPerLane; ++i) {
+                const int r = lane + 32 * i;
+                const int item_row = row0 + r, po = item_row / g;
+                hh[i] = item_row - po * g;
+                occ[i] = r >= n_rows ? 0 : a.prefill ? occ_off + po : __ldcg(a.occ + occ_off + po);
+            }
             for (int t = lane; t < n_tiles; t += 32) c.tiles[q][t] = word_at(a.tiles, a.w_tiles, tile_off + t);
+#pragma unroll
+            for (int i = 0; i < kRowsPerLane; ++i) {
+                if (!check(in_range(occ[i], a.ext.n), a.err)) occ[i] = 0;
+                src_row[i] = (uint32_t)occ[i] * (uint32_t)a.hq + (uint32_t)(kvh * g + hh[i]);
+            }
+        }
         if (lane < kUnitWords) reinterpret_cast<volatile int*>(c.desc[q])[lane] = word;
         if (lane == kUnitWords || lane == kUnitWords + 1)
             reinterpret_cast<volatile int*>(c.desc[q])[lane] =
@@ -1842,41 +1867,24 @@ __device__ void tc_fetch(const DecodeArgs& a, const ParamWords<CAP>& p, CtlTc& c
             if (lane == 0) rearm(a);
             return;
         }
-        const int occ_off = __shfl_sync(0xffffffffu, word, U_OCC_OFF);
-        const int row0 = __shfl_sync(0xffffffffu, word, U_ROW0);
-        const int n_rows = __shfl_sync(0xffffffffu, word, U_N_ROWS);
-        const int kvh = __shfl_sync(0xffffffffu, word, U_KVH);
         // the previous unit's Q.K^T MMAs have read the buffer
         if (!mbar_wait(smem_u32(&c.qempty), (k & 1) ^ 1)) note_timeout(a, c, 2);
-        constexpr int CH = HD / 8;  // 16-byte chunks per row
-        const int g = a.group;
-        // lane = query row (rows lane, lane + 32, ...): its source row is
-        // found once -- prefill schedules list query rows in order
-        // (occurrence = query index), decode looks the occurrence up, all
-        // lookups in flight together -- then its CH chunks go out as 16-byte
-        // async copies straight into the swizzled layout, offsets known at
-        // compile time, every copy of the tile in flight at once
-        constexpr int kRowsPerLane = kTcRows / 32;
-        const bool in_order = a.prefill != 0;
-        int64_t src_off[kRowsPerLane];
-#pragma unroll
-        for (int i = 0; i < kRowsPerLane; ++i) {
-            const int r = lane + 32 * i;
-            const int item_row = row0 + r, po = item_row / g, hh = item_row - po * g;
-            int occ = r >= n_rows ? 0 : in_order ? occ_off + po : __ldcg(a.occ + occ_off + po);
-            if (!check(in_range(occ, a.ext.n), a.err)) occ = 0;
-            src_off[i] = ((int64_t)occ * a.hq + kvh * g + hh) * HD;
-        }
+        // 16-byte async copies straight into the swizzled layout, eight lanes
+        // to a 128-byte line (a row per lane asked for 32 lines an instruction
+        // and every 32-byte sector twice: prefill of 64 prompts 325 us against
+        // 311, of a 717-token prompt 17.8 / 17.2, decode over a 2k prefix 306.9
+        // / 304.8)
         const uint32_t q_base = smem_u32(qbuf);
+        const int sub = lane >> 3, ch = lane & 7;
 #pragma unroll
-        for (int i = 0; i < kRowsPerLane; ++i) {
-            const int r = lane + 32 * i;
-            if (r >= n_rows) break;
-            const uint16_t* src = a.q + src_off[i];
-            const uint32_t dst = q_base + r * 128, x = r & 7;
+        for (int i = 0; i < kTcRows / 4; ++i) {
+            const int r = 4 * i + sub;
+            const uint32_t from = __shfl_sync(0xffffffffu, src_row[i >> 3], r & 31);
+            if (r >= n_rows) continue;
+            const uint16_t* src = a.q + (uint64_t)from * HD + ch * 8;
+            const uint32_t dst = q_base + r * 128 + ((ch ^ (r & 7)) << 4);
 #pragma unroll
-            for (int ch = 0; ch < CH; ++ch)
-                cp_async16(dst + (ch >> 3) * (kTcRows * 128) + (((ch & 7) ^ x) << 4), src + ch * 8);
+            for (int h = 0; h < HD / 64; ++h) cp_async16(dst + h * (kTcRows * 128), src + h * 64);
         }
         cp_async_wait_all();
         fence_proxy_async();  // the copies -> visible to the tensor core
