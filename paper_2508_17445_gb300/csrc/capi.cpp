@@ -728,11 +728,42 @@ tp_status tp_prefill(tp_tree* t, const tp_node* nodes, const int32_t* n_queries,
 }  // extern "C"
 
 namespace {
+// Device address of page-locked host memory, null for any other.
+void* mapped_host(void* p, uintptr_t align) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return at.type == cudaMemoryTypeHost && at.devicePointer && aligned(at.devicePointer, align) ? at.devicePointer
+                                                                                                 : nullptr;
+}
+
+// Whether a decode call's merge writes its results to page-locked host memory
+// itself (each row once, whole lines) instead of leaving them to a download.
+// A caller that waits after each call saves the download and the hop to its
+// stream (256 leaves 149 us a call -> 141, 8 leaves 46 -> 38); back to back,
+// downloads overlap the next call while the merge's stores to the host do not
+// (256 leaves 94 us a call against 102, 1024 leaves 329 / 356, but 16 leaves,
+// 115 KB, 20.2 either way). So: small results always, others when the call
+// before has finished.
+constexpr int64_t kDirectBytes = 128 << 10;
+
+bool write_direct(const tp_tree* t, int64_t o_bytes) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(t->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    if (o_bytes <= kDirectBytes || t->hp_calls == 0) return true;
+    const cudaError_t e = cudaEventQuery(t->hp_done[(t->hp_calls - 1) & 1]);
+    if (e != cudaSuccess) cudaGetLastError();  // (not ready is an error code too)
+    return e == cudaSuccess;
+}
+
 // One host-buffer call: upload Q into staging slot b once the attention that
 // last read that slot has finished, run the attention there once the upload
 // has landed and the slot's previous results have been downloaded, then
-// download O and LSE. Consecutive calls alternate slots, so a call's upload
-// and download overlap the neighbouring calls' attention.
+// download O and LSE (o_bytes == 0: the kernels write them to the host
+// themselves). Consecutive calls alternate slots, so a call's upload and
+// download overlap the neighbouring calls' attention.
 template <typename Run>
 tp_status run_host(tp_tree* t, int64_t q_bytes, int64_t o_bytes, int64_t lse_bytes, const void* Qh, void* Oh,
                    float* Lh, Run run) {
@@ -761,10 +792,17 @@ tp_status run_host(tp_tree* t, int64_t q_bytes, int64_t o_bytes, int64_t lse_byt
     if (e == cudaSuccess) e = cudaEventRecord(t->hp_up[b], t->hp_h2d);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(t->stream, t->hp_up[b], 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(t->stream, t->hp_down[b], 0);
+    if (e == cudaSuccess && o_bytes == 0)  // nor may an earlier download land after these kernels' results
+        e = cudaStreamWaitEvent(t->stream, t->hp_down[b ^ 1], 0);
     if (e != cudaSuccess) return cuda_fail(t, e, "query upload");
     st = run(t->hp_q[b], t->hp_o[b], (float*)t->hp_lse[b]);
     if (st != TP_OK) return st;
     e = cudaEventRecord(t->hp_done[b], t->stream);
+    if (o_bytes == 0) {
+        if (e != cudaSuccess) return cuda_fail(t, e, "cudaEventRecord");
+        ++t->hp_calls;
+        return TP_OK;
+    }
     if (e == cudaSuccess) e = cudaStreamWaitEvent(t->hp_d2h, t->hp_done[b], 0);
     if (e == cudaSuccess) e = cudaMemcpyAsync(Oh, t->hp_o[b], (size_t)o_bytes, cudaMemcpyDeviceToHost, t->hp_d2h);
     if (e == cudaSuccess) e = cudaMemcpyAsync(Lh, t->hp_lse[b], (size_t)lse_bytes, cudaMemcpyDeviceToHost, t->hp_d2h);
@@ -787,8 +825,13 @@ tp_status tp_decode_host(tp_tree* t, const tp_node* leaves, int32_t n, const voi
     if (!t->cfg.pool) return fail(t, TP_ERR_INVALID_ARG, "metadata-only tree cannot decode");
     if (!Q_host || !O_host || !LSE_host) return fail(t, TP_ERR_INVALID_ARG, "Q/O/LSE host pointer is NULL");
     const int64_t row = (int64_t)t->cfg.num_q_heads * t->cfg.head_dim;
-    return run_host(t, n * row * 2, n * row * 2, (int64_t)n * t->cfg.num_q_heads * 4, Q_host, O_host, LSE_host,
-                    [&](const void* Q, void* O, float* LSE) { return tp_decode_ex(t, leaves, n, Q, O, LSE, flags); });
+    void* O_dev = mapped_host(O_host, 16);
+    float* LSE_dev = (float*)mapped_host(LSE_host, 4);
+    const bool direct = O_dev && LSE_dev && write_direct(t, n * row * 2);
+    return run_host(t, n * row * 2, direct ? 0 : n * row * 2, direct ? 0 : (int64_t)n * t->cfg.num_q_heads * 4, Q_host,
+                    O_host, LSE_host, [&](const void* Q, void* O, float* LSE) {
+                        return tp_decode_ex(t, leaves, n, Q, direct ? O_dev : O, direct ? LSE_dev : LSE, flags);
+                    });
 }
 
 tp_status tp_prefill_host(tp_tree* t, const tp_node* nodes, const int32_t* n_queries, int32_t n, const void* Q_host,
