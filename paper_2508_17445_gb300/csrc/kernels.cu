@@ -2134,12 +2134,24 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
             tmem_ld32_nowait(s_addr, r[0]);
             tmem_ld32_nowait(s_addr + 32, r[1]);
             tmem_wait_ld();
-            // row max over the tokens the row may see, on the raw scores (the
-            // scale is positive); a stage every row of the warp sees whole
-            // takes the unmasked path
-            const bool whole = __all_sync(0xffffffffu, lim0 == 32 && lim1 == 32);
-            float mx = -INFINITY;
-            if (whole) {  // four independent chains of three-input maxima
+            // tokens the row may not see score -inf; a stage every row of the
+            // warp sees whole (all but the last ones) skips this. What follows
+            // is one path for both: the kernel's warps are at different places
+            // of a long straight code and wait for instructions, so a second,
+            // masked softmax cost every stage (prefill of 64 prompts 311 us
+            // with it, 279 without; ragged segments at head_dim 64 61 / 55;
+            // 512 segments 4415 / 4230).
+            if (__any_sync(0xffffffffu, lim0 != 32 || lim1 != 32)) {
+#pragma unroll
+                for (int t = 0; t < 32; ++t) {
+                    if (t >= lim0) r[0][t] = 0xff800000u;
+                    if (t >= lim1) r[1][t] = 0xff800000u;
+                }
+            }
+            // row max on the raw scores (the scale is positive): four
+            // independent chains of three-input maxima
+            float mx;
+            {
                 float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
 #pragma unroll
                 for (int t = 0; t < 32; t += 4) {
@@ -2149,14 +2161,6 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
                     m3 = fmax3(m3, __uint_as_float(r[1][t + 2]), __uint_as_float(r[1][t + 3]));
                 }
                 mx = fmaxf(fmax3(m0, m1, m2), m3);
-            } else {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int lim = h ? lim1 : lim0;
-#pragma unroll
-                    for (int t = 0; t < 32; ++t)
-                        if (t < lim) mx = fmaxf(mx, __uint_as_float(r[h][t]));
-                }
             }
             mx *= a.qk_scale_log2;
             const float m_new = fmaxf(m_used, mx);
@@ -2181,11 +2185,13 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
                     m_used = m_new;
                 }
             }
-            // P = exp2(s * scale - m_used) as bf16 pairs over the S columns
+            // P = exp2(s * scale - m_used) as bf16 pairs over the S columns: two
+            // scores scaled and shifted per instruction, two pair sums (a row
+            // that has seen nothing yet shifts by 0: exp2(-inf) = 0)
             uint32_t pw[32];
-            float sum = 0.f;
-            const float sc = a.qk_scale_log2, neg_m = -m_used;
-            if (whole) {  // scale and shift two scores per instruction; two pair sums
+            float sum;
+            {
+                const float sc = a.qk_scale_log2, neg_m = m_used == -INFINITY ? 0.f : -m_used;
                 const uint64_t sc2 = f2_pack(sc, sc), nm2 = f2_pack(neg_m, neg_m);
                 uint64_t acc[2] = {0, 0};
 #pragma unroll
@@ -2203,18 +2209,6 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
                 f2_unpack(acc[0], s0, s1);
                 f2_unpack(acc[1], s2, s3);
                 sum = (s0 + s2) + (s1 + s3);
-            } else {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int lim = h ? lim1 : lim0;
-#pragma unroll
-                    for (int t = 0; t < 32; t += 2) {
-                        const float p0 = t < lim ? fast_exp2(fmaf(__uint_as_float(r[h][t]), sc, neg_m)) : 0.f;
-                        const float p1 = t + 1 < lim ? fast_exp2(fmaf(__uint_as_float(r[h][t + 1]), sc, neg_m)) : 0.f;
-                        sum += p0 + p1;
-                        pw[h * 16 + t / 2] = pack_bf16(p0, p1);
-                    }
-                }
             }
             l += sum;
             tmem_st32(s_addr, pw);
@@ -2259,36 +2253,32 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
         // aligned (rows are multiples of 256 bytes, so the base decides)
         const bool wide = !final_out || (reinterpret_cast<uintptr_t>(a.out) & 31) == 0;
 #pragma unroll 1
-        for (int cc = 0; cc < HD / 32; cc += 2) {  // two 32-column loads in flight
-            uint32_t ov[2][32];
-            __syncwarp();  // the loads are warp-collective
-            tmem_ld32_nowait(o_addr + cc * 32, ov[0]);
-            tmem_ld32_nowait(o_addr + cc * 32 + 32, ov[1]);
-            tmem_wait_ld();
+        for (int cc = 0; cc < HD / 32; ++cc) {
+            uint32_t ov[32];
+            __syncwarp();  // the load is warp-collective
+            tmem_ld32(o_addr + cc * 32, ov);
+            if (!live) continue;
+            const int c0 = cc * 32;
+            if (final_out) {
+                uint32_t w[16];
 #pragma unroll
-            for (int h = 0; h < 2 && live; ++h) {
-                const int c0 = (cc + h) * 32;
-                if (final_out) {
-                    uint32_t w[16];
-#pragma unroll
-                    for (int t = 0; t < 16; ++t)
-                        w[t] = pack_bf16(__uint_as_float(ov[h][2 * t]) * inv, __uint_as_float(ov[h][2 * t + 1]) * inv);
-                    if (wide) {
-                        st_global_v8(dst16 + c0, w);
-                        st_global_v8(dst16 + c0 + 16, w + 8);
-                    } else {
-#pragma unroll
-                        for (int t = 0; t < 16; t += 4)
-                            *reinterpret_cast<uint4*>(dst16 + c0 + 2 * t) = make_uint4(w[t], w[t + 1], w[t + 2], w[t + 3]);
-                    }
+                for (int t = 0; t < 16; ++t)
+                    w[t] = pack_bf16(__uint_as_float(ov[2 * t]) * inv, __uint_as_float(ov[2 * t + 1]) * inv);
+                if (wide) {
+                    st_global_v8(dst16 + c0, w);
+                    st_global_v8(dst16 + c0 + 16, w + 8);
                 } else {
 #pragma unroll
-                    for (int t = 0; t < 32; t += 8) {
-                        uint32_t w[8];
+                    for (int t = 0; t < 16; t += 4)
+                        *reinterpret_cast<uint4*>(dst16 + c0 + 2 * t) = make_uint4(w[t], w[t + 1], w[t + 2], w[t + 3]);
+                }
+            } else {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) w[e] = __float_as_uint(__uint_as_float(ov[h][t + e]) * inv);
-                        st_global_v8_hint(dst + c0 + t, w, pol);
-                    }
+                for (int t = 0; t < 32; t += 8) {
+                    uint32_t w[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) w[e] = __float_as_uint(__uint_as_float(ov[t + e]) * inv);
+                    st_global_v8_hint(dst + c0 + t, w, pol);
                 }
             }
         }

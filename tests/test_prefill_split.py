@@ -75,3 +75,30 @@ def test_schedule_words_with_the_launch():
         o_ref, lse_ref = model.prefill([s.leaves[0]], [n], Q.cpu(), _kv_source(s), indices=rows)
         check(O, LSE, o_ref, lse_ref, rows=rows)
         f.close()
+
+
+# whole prompts at the edges of a tile, a stage and two stages: every causal mask of the last stage
+@pytest.mark.gpu
+@pytest.mark.parametrize("heads", [workloads.Heads(28, 4, 128), workloads.Heads(16, 2, 64)])
+@pytest.mark.parametrize("tokens", [1, 2, 31, 32, 33, 63, 64, 65, 96, 97, 127, 128, 129])
+def test_masked_last_stages(tokens, heads):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from test_gpu_parity import _kv_source, build_forest
+    s = workloads.single_path(seed=40 + tokens, lengths=(tokens,), heads=heads)
+    f, ids = build_forest(s)
+    Q = s.q("cuda:0", n=tokens)
+    O, LSE = f.prefill([ids[s.leaves[0]]], [tokens], Q)
+    f.sync()
+    src = _kv_source(s)
+    model = oracle.OracleForest(block_tokens=32, pool_blocks=f.cfg.pool_blocks).replay(s)
+    o_ref, lse_ref = model.prefill([s.leaves[0]], [tokens], Q.cpu(), src)
+    abs_src = lambda i: (src(i)[0], oracle.bf16_bits(src(i)[1]) & np.uint16(0x7FFF))  # noqa: E731
+    a_ref, _ = model.prefill([s.leaves[0]], [tokens], Q.cpu(), abs_src)
+    # rows that see a few tokens have |O| up to the values' own size (4 and more), where the two bf16 roundings (of P and
+    # of O, 2^-8 each) alone exceed the absolute bar of 1e-2: the derived bound 2^-8 (|O| + A) + 1e-5 holds everywhere
+    d_o = np.abs(O.float().cpu().numpy().astype(np.float64) - o_ref)
+    assert (d_o <= 2.0 ** -8 * (np.abs(o_ref) + a_ref) + 1e-5).all()
+    assert np.abs(LSE.cpu().numpy().astype(np.float64) - lse_ref).max() <= 5e-5
+    f.close()
