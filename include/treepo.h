@@ -520,8 +520,8 @@ tp_status tp_synth_tokens(tp_tree* tree, uint64_t seed, tp_node node, int32_t po
  * parent table was malformed (an id out of range or a cycle; the affected
  * trajectories are rejected). workspace: device, 8-byte aligned, at least
  * tp_advantage_workspace_bytes(n_nodes, n_out) bytes. Fp64 accumulation,
- * one cooperative kernel (ancestor sums, sub-group means and A_i, statistics),
- * or four kernels past 38912 outputs; asynchronous on cuda_stream; calls
+ * one kernel (ancestor sums, sub-group means and A_i, statistics; one cluster
+ * up to 1024 outputs, a cooperative grid up to 38912) or four; asynchronous on cuda_stream; calls
  * sharing a workspace must not overlap. Errors (tp_last_error(NULL)):
  * TP_ERR_INVALID_ARG, TP_ERR_CUDA.
  */

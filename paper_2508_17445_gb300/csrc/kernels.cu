@@ -635,9 +635,12 @@ __global__ void __launch_bounds__(kAdvAbarThreads) advantage_abar_kernel(const A
 //    taken out of A_i already, so their own mean stays below their spread and
 //    E[A^2] - E[A]^2 does not cancel.
 // 1024 trajectories, 10k nodes: four launches 32 us a call, one with plain
-// divisions and two-pass statistics 30.7, this one 19.2 (three grid
-// barriers of ~1.8 us, the walk 1.8, the means ~2).
-constexpr int kAdvCta = 128;    // threads of a CTA; the first per_cta of them hold an output each
+// divisions and two-pass statistics 30.7, this one over a grid 19.2 (three
+// grid barriers of ~1.8 us, the walk 1.8, the means ~2), in one cluster
+// (CLUSTER: up to 1024 outputs, hardware barriers, a warp of outputs on each
+// sub-partition of eight SMs) 15.4.
+constexpr int kAdvCta = 128;    // outputs a CTA may hold: one for each of its first per_cta threads
+constexpr int kAdvClusterThreads = 512, kAdvClusterCtas = 8;  // (the other threads help to clear the tables)
 constexpr int kAdvChain = 64;   // ancestors kept; deeper ones are walked again
 constexpr int kAdvMaxCtas = 2 * 152;
 constexpr int kInvTable = 256;
@@ -658,11 +661,23 @@ __device__ __forceinline__ double div_small(double x, int n) {
     return fma(fma(-q, (double)n, x), y, q);
 }
 
-__global__ void __launch_bounds__(kAdvCta) advantage_kernel(const AdvantageArgs a, int per_cta) {
+template <bool CLUSTER>
+__global__ void __launch_bounds__(CLUSTER ? kAdvClusterThreads : kAdvCta)
+    advantage_kernel(const AdvantageArgs a, int per_cta) {
+    constexpr int kThreads = CLUSTER ? kAdvClusterThreads : kAdvCta;
     __shared__ int32_t chain[kAdvChain][kAdvCta];
-    const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    auto sync_all = [] {
+        if constexpr (CLUSTER)
+            cooperative_groups::this_cluster().sync();
+        else
+            cooperative_groups::this_grid().sync();
+    };
+    if constexpr (CLUSTER) {  // (launched under its predecessor)
+        dep_trigger();
+        dep_wait();
+    }
     const AdvWs w = adv_ws(a);
-    for (int64_t x = (int64_t)blockIdx.x * kAdvCta + threadIdx.x; x < a.n_nodes; x += (int64_t)gridDim.x * kAdvCta) {
+    for (int64_t x = (int64_t)blockIdx.x * kThreads + threadIdx.x; x < a.n_nodes; x += (int64_t)gridDim.x * kThreads) {
         w.cnt[x] = 0;
         w.sum[x] = 0.0;
         w.kmin[x] = 0xffffffffu;
@@ -696,7 +711,7 @@ __global__ void __launch_bounds__(kAdvCta) advantage_kernel(const AdvantageArgs 
         }
     }
     const int kept = min(depth, kAdvChain);
-    grid.sync();  // tables clear
+    sync_all();  // tables clear
     if (mine) {
         int32_t x = -1;
         for (int k = 0; k < depth; ++k) {
@@ -711,7 +726,7 @@ __global__ void __launch_bounds__(kAdvCta) advantage_kernel(const AdvantageArgs 
             atomicMax(&w.kmax[root], reward_key(rf));
         }
     }
-    grid.sync();  // sums complete
+    sync_all();  // sums complete
     double s = 0.0;
     const bool accepted = mine && !bad && depth > 0 && __ldcg(&w.kmin[root]) != __ldcg(&w.kmax[root]);
     if (accepted) {
@@ -753,7 +768,7 @@ __global__ void __launch_bounds__(kAdvCta) advantage_kernel(const AdvantageArgs 
             }
         }
     }
-    grid.sync();  // totals complete
+    sync_all();  // totals complete
     const int n = __ldcg(&w.flags[1]);
     const double inv_n = n > 0 ? div_small(1.0, n) : 0.0;
     const double mean = __ldcg(&w.tot[0]) * inv_n;
@@ -2781,19 +2796,32 @@ int64_t advantage_ws_bytes(int64_t n_nodes, int64_t n_out) {
 
 cudaError_t launch_advantage(const AdvantageArgs& a, cudaStream_t s) {
     if (a.n_out > 0 && a.n_out <= kAdvMaxCtas * kAdvCta) {
-        // one warp of outputs per CTA while two CTAs per SM hold them all
-        // (fp64 units and walk latency spread over the SMs), then more
-        const int per_cta = (int)(((a.n_out + kAdvMaxCtas - 1) / kAdvMaxCtas + 31) / 32 * 32);
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeCooperative;
-        attr.val.cooperative = 1;
+        const bool cluster = a.n_out <= kAdvClusterCtas * kAdvCta;
+        const int ctas = cluster ? kAdvClusterCtas : kAdvMaxCtas;
+        // one warp of outputs per CTA while the CTAs hold them all (fp64 units
+        // and walk latency spread over the SMs), then more
+        const int per_cta = (int)(((a.n_out + ctas - 1) / ctas + 31) / 32 * 32);
+        cudaLaunchAttribute attr[2] = {};
         cudaLaunchConfig_t cfg{};
+        cfg.stream = s;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cluster) {
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = kAdvClusterCtas;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[1].val.programmaticStreamSerializationAllowed = 1;
+            cfg.numAttrs = 2;
+            cfg.gridDim = dim3(kAdvClusterCtas);
+            cfg.blockDim = dim3(kAdvClusterThreads);
+            return cudaLaunchKernelEx(&cfg, advantage_kernel<true>, a, per_cta);
+        }
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
         cfg.gridDim = dim3((a.n_out + per_cta - 1) / per_cta);
         cfg.blockDim = dim3(kAdvCta);
-        cfg.stream = s;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, advantage_kernel, a, per_cta);
+        return cudaLaunchKernelEx(&cfg, advantage_kernel<false>, a, per_cta);
     }
     const int init_grid = (int)std::min<int64_t>(std::max<int64_t>(1, (a.n_nodes + kAdvThreads - 1) / kAdvThreads),
                                                  152 * 8);

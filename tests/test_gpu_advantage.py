@@ -1,8 +1,8 @@
-"""The tree advantage over the sizes where its launch changes: one CTA and
-several, the last output of a CTA, one to four warps of outputs per CTA, and
-more outputs than the cooperative launch has threads (then four launches);
-paths deeper than the ancestors a thread keeps. Oracle and tolerance of
-test_gpu_rollout.py (fp64 accumulation, fp32 output: 1e-6 (|adv| + 1))."""
+"""The tree advantage over the sizes where its launch changes: one cluster (up
+to 1024 outputs) and a grid, the last output of a CTA, one to four warps of
+outputs per CTA, and more outputs than the grid has threads (then four
+launches); paths deeper than the ancestors a thread keeps. Oracle and tolerance
+of test_gpu_rollout.py (fp64 accumulation, fp32 output: 1e-6 (|adv| + 1))."""
 import numpy as np
 import pytest
 
@@ -31,7 +31,7 @@ def flat_trees(n_out, width, depth, seed):
     return np.array(parent, np.int32), leaf, rng.random(n_out).round(2)
 
 
-@pytest.mark.parametrize("n_out", [1, 2, 31, 32, 33, 128, 9728, 9729, 19457, 38912, 38913])
+@pytest.mark.parametrize("n_out", [1, 2, 31, 32, 33, 128, 256, 257, 1023, 1024, 1025, 9728, 9729, 19457, 38912, 38913])
 def test_outputs_per_launch(n_out):
     check_advantage(*flat_trees(n_out, 16, 3, n_out))
 
@@ -39,6 +39,7 @@ def test_outputs_per_launch(n_out):
 @pytest.mark.parametrize("depth", [1, 63, 64, 65, 66, 200])
 def test_deep_paths(depth):
     check_advantage(*flat_trees(100, 7, depth, depth))
+    check_advantage(*flat_trees(1100, 7, depth, depth))
 
 
 def test_all_equal_and_negative_rewards():
