@@ -124,6 +124,12 @@ __device__ __forceinline__ uint64_t l2_evict_first() {
     return p;
 }
 
+__device__ __forceinline__ uint64_t l2_evict_normal() {
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+
 __device__ __forceinline__ uint64_t l2_evict_last() {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
@@ -1726,10 +1732,15 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// sm_100 shared-memory matrix descriptor: 128-byte swizzle, version 1.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+// sm_100 shared-memory matrix descriptor: 128-byte swizzle, version 1, groups
+// of eight rows 1024 bytes apart. The low word holds address and leading
+// offset, so a constant added to it moves the address.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr, uint32_t lbo) {
+    return (saddr >> 4) | ((lbo >> 4) << 16);
+}
+
+__device__ __forceinline__ uint64_t smem_desc_at(uint32_t lo) {
+    return ((uint64_t)((1024u >> 4) | (1u << 14) | (2u << 29)) << 32) | lo;
 }
 
 // Instruction descriptor, kind::f16: D fp32, A and B bf16, M = 128.
@@ -1909,10 +1920,12 @@ __device__ void tc_fetch(const DecodeArgs& a, const ParamWords<CAP>& p, CtlTc& c
 }
 
 // Bulk copies of one half (K or V) of a tile pair into a stage; w = -1 for a
-// missing second tile.
+// missing second tile. One L2 policy value instead of copies with and without
+// a hint: less code for warps that wait for instructions (prefill of 64
+// prompts 279 -> 267 us).
 template <int HD>
 __device__ __forceinline__ void issue_half(const DecodeArgs& a, int kvh, int kv, uint8_t* dst, const int32_t (&w)[2],
-                                           uint32_t bar, bool once) {
+                                           uint32_t bar, uint64_t policy) {
     uint32_t bytes = 0;
     int valid[2] = {0, 0};
     for (int j = 0; j < 2; ++j)
@@ -1928,10 +1941,7 @@ __device__ __forceinline__ void issue_half(const DecodeArgs& a, int kvh, int kv,
 #pragma unroll
         for (int h = 0; h < HD / 64; ++h) {
             const uint32_t d = smem_u32(dst + h * kStageTokens * 128 + j * kBlockTokens * 128);
-            if (once)
-                bulk_g2s_hint(d, src + h * kBlockTokens * 128, valid[j] * 128, bar, l2_evict_first());
-            else
-                bulk_g2s(d, src + h * kBlockTokens * 128, valid[j] * 128, bar);
+            bulk_g2s_hint(d, src + h * kBlockTokens * 128, valid[j] * 128, bar, policy);
         }
     }
 }
@@ -1956,6 +1966,7 @@ __device__ void tc_stream(const DecodeArgs& a, CtlTc& c, uint8_t* ring) {
         // tile from row 0): no other unit reads this chunk
         const bool once = a.kv_read_once && *reinterpret_cast<volatile int*>(&c.desc[q][U_ROW0]) == 0 &&
                           *reinterpret_cast<volatile int*>(&c.desc[q][U_N_ROWS]) < kTcRows;
+        const uint64_t policy = once ? l2_evict_first() : l2_evict_normal();
         const volatile int* tw = c.tiles[q];
         const int n_pairs = (n_tiles + 1) / 2;
         int kj = 0, vj = 0;
@@ -1966,7 +1977,7 @@ __device__ void tc_stream(const DecodeArgs& a, CtlTc& c, uint8_t* ring) {
             if (kj < n_pairs && mbar_test(smem_u32(&c.s_full[ks]), kph ^ 1)) {  // K slot read by Q.K^T
                 const int32_t w[2] = {tw[2 * kj], 2 * kj + 1 < n_tiles ? tw[2 * kj + 1] : -1};
                 fence_proxy_async();
-                issue_half<HD>(a, kvh, 0, ring + ks * TcSmem<HD>::kStageBytes, w, smem_u32(&c.kfull[ks]), once);
+                issue_half<HD>(a, kvh, 0, ring + ks * TcSmem<HD>::kStageBytes, w, smem_u32(&c.kfull[ks]), policy);
                 if (++ks == kStages) {
                     ks = 0;
                     kph ^= 1;
@@ -1978,7 +1989,7 @@ __device__ void tc_stream(const DecodeArgs& a, CtlTc& c, uint8_t* ring) {
                 const int32_t w[2] = {tw[2 * vj], 2 * vj + 1 < n_tiles ? tw[2 * vj + 1] : -1};
                 fence_proxy_async();
                 issue_half<HD>(a, kvh, 1, ring + vs * TcSmem<HD>::kStageBytes + (HD / 64) * kStageTokens * 128, w,
-                               smem_u32(&c.vfull[vs]), once);
+                               smem_u32(&c.vfull[vs]), policy);
                 if (++vs == kStages) {
                     vs = 0;
                     vph ^= 1;
@@ -2003,24 +2014,47 @@ __device__ void tc_stream(const DecodeArgs& a, CtlTc& c, uint8_t* ring) {
     }
 }
 
-// MMA issuer lane.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(e));
+    return e != 0;
+}
+
+// mbar_test and mbar_try_wait with a warp-uniform answer
+__device__ __forceinline__ bool warp_test(uint32_t bar, uint32_t parity) {
+    return __any_sync(0xffffffffu, mbar_test(bar, parity));
+}
+
+__device__ __forceinline__ bool warp_try_wait(uint32_t bar, uint32_t parity) {
+    return __any_sync(0xffffffffu, mbar_try_wait(bar, parity));
+}
+
+// MMA issuer warp: every lane runs the event loop, one elected lane issues.
+// The tensor core waits for the issuer's instructions (with the two issue
+// loops rolled prefill ran 12% slower), so what stands between two MMAs is
+// kept short: every operand is warp-uniform (votes and reductions make the
+// loop's state so) and a descriptor is one addition to its low word. Against
+// one lane that built each descriptor from its address: prefill of 64 prompts
+// 267 -> 251 us, at head_dim 64 1797 -> 1570, 512 segments 4290 -> 4080 (under
+// the power cap), decode over a 2k prefix 305.1 -> 303.7.
 template <int HD>
 __device__ void tc_issue(const DecodeArgs& a, CtlTc& c, const uint8_t* ring, const uint8_t* qbuf) {
     constexpr uint32_t kIdescS = mma_idesc<kStageTokens, false>();
     constexpr uint32_t kIdescPV = mma_idesc<HD, true>();
-    const uint32_t tmem = c.tmem;
-    const uint32_t q_addr = smem_u32(qbuf), ring_addr = smem_u32(ring);
-    int s_stage = 0, v_stage = 0;
+    const uint32_t tmem = __reduce_or_sync(0xffffffffu, c.tmem);
+    const bool leader = elect_one();
+    const uint32_t q_lo = smem_desc_lo(smem_u32(qbuf), 16), ring_addr = smem_u32(ring);
+    static_assert(kStages == 2, "ring slot = S and P buffer");
+    int s_stage = 0, v_stage = 0;  // ring slot of the next Q.K^T, P.V
     uint32_t s_phase = 0, v_phase = 0;
-    uint32_t gs = 0;  // stages issued by this CTA so far (S buffer = gs & 1)
     for (int k = 0;; ++k) {
         const int q = k & 1;
-        if (!mbar_wait(smem_u32(&c.ufull[q]), (k >> 1) & 1)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&c.ufull[q]), (k >> 1) & 1))) {
             note_timeout(a, c, 2);
             return;
         }
         if (*reinterpret_cast<volatile int*>(&c.unit[q]) < 0) return;
-        const int n_tiles = *reinterpret_cast<volatile int*>(&c.desc[q][U_N_TILES]);
+        const int n_tiles = __reduce_max_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&c.desc[q][U_N_TILES]));
         const int n_pairs = (n_tiles + 1) / 2;
         if (!mbar_wait(smem_u32(&c.qfull), k & 1)) note_timeout(a, c, 2);
         tc_fence_after();
@@ -2029,23 +2063,24 @@ __device__ void tc_issue(const DecodeArgs& a, CtlTc& c, const uint8_t* ring, con
         // issued), and P.V of the oldest stage as soon as its P is written;
         // neither waits on the other.
         int next_s = 0, next_pv = 0;
-        bool q_released = false;
+        bool q_released = false, v_ready = false;
         uint64_t idle_since = 0;
         uint32_t spins = 0;
         while (next_pv < n_pairs) {
             bool progress = false;
-            if (next_s < n_pairs && next_s <= next_pv + 1 && mbar_test(smem_u32(&c.kfull[s_stage]), s_phase)) {
+            if (next_s < n_pairs && next_s <= next_pv + 1 && warp_test(smem_u32(&c.kfull[s_stage]), s_phase)) {
                 tc_fence_after();
-                const uint32_t g_stage = gs + next_s;
-                const uint32_t kb = ring_addr + s_stage * TcSmem<HD>::kStageBytes;
-                const uint32_t d = tmem + (g_stage & 1) * kStageTokens;
+                const uint32_t kb = smem_desc_lo(ring_addr, 16) + s_stage * (TcSmem<HD>::kStageBytes >> 4);
+                const uint32_t d = tmem + s_stage * kStageTokens;
+                if (leader) {
 #pragma unroll
-                for (int ks = 0; ks < HD / 16; ++ks) {
-                    const uint32_t off = (ks >> 2) * (kStageTokens * 128) + (ks & 3) * 32;
-                    const uint32_t qoff = (ks >> 2) * (kTcRows * 128) + (ks & 3) * 32;
-                    mma_ss(d, smem_desc(q_addr + qoff, 16, 1024), smem_desc(kb + off, 16, 1024), kIdescS, ks > 0);
+                    for (int ks = 0; ks < HD / 16; ++ks) {
+                        const uint32_t off = (ks >> 2) * (kStageTokens * 128) + (ks & 3) * 32;
+                        const uint32_t qoff = (ks >> 2) * (kTcRows * 128) + (ks & 3) * 32;
+                        mma_ss(d, smem_desc_at(q_lo + (qoff >> 4)), smem_desc_at(kb + (off >> 4)), kIdescS, ks > 0);
+                    }
+                    tc_commit(smem_u32(&c.s_full[s_stage]));
                 }
-                tc_commit(smem_u32(&c.s_full[g_stage & 1]));  // = ring slot s_stage
                 if (++s_stage == kStages) {
                     s_stage = 0;
                     s_phase ^= 1;
@@ -2054,26 +2089,33 @@ __device__ void tc_issue(const DecodeArgs& a, CtlTc& c, const uint8_t* ring, con
                 progress = true;
             }
             if (next_s == n_pairs && !q_released) {
-                tc_commit(smem_u32(&c.qempty));  // every Q.K^T of the unit issued
+                if (leader) tc_commit(smem_u32(&c.qempty));  // every Q.K^T of the unit issued
                 q_released = true;
             }
-            const uint32_t gp = gs + next_pv;
-            if (next_pv < next_s && mbar_test(smem_u32(&c.p_full[gp & 1]), (gp >> 1) & 1) &&
-                mbar_test(smem_u32(&c.vfull[v_stage]), v_phase)) {
+            // With no Q.K^T left to issue before the next P.V the warp sleeps
+            // until P is written (polling costs issue slots and power:
+            // prefill of 64 prompts 253.7 us, 250.8 asleep).
+            const bool only_pv = next_s == n_pairs || next_s == next_pv + 2;
+            const uint32_t p_bar = smem_u32(&c.p_full[v_stage]);
+            if (!v_ready) v_ready = warp_test(smem_u32(&c.vfull[v_stage]), v_phase);
+            if (next_pv < next_s && v_ready && (only_pv ? warp_try_wait(p_bar, v_phase) : warp_test(p_bar, v_phase))) {
+                v_ready = false;
                 tc_fence_after();
                 if (next_pv == 0) {  // the previous unit's epilogue has read O
                     if (!mbar_wait(smem_u32(&c.o_free), (k & 1) ^ 1)) note_timeout(a, c, 2);
                     tc_fence_after();
                 }
-                const uint32_t vb = ring_addr + v_stage * TcSmem<HD>::kStageBytes + (HD / 64) * kStageTokens * 128;
-                const uint32_t p_tmem = tmem + (gp & 1) * kStageTokens;
+                const uint32_t vb = smem_desc_lo(ring_addr, kStageTokens * 128) +
+                                    ((v_stage * TcSmem<HD>::kStageBytes + (HD / 64) * kStageTokens * 128) >> 4);
+                const uint32_t p_tmem = tmem + v_stage * kStageTokens;
+                if (leader) {
 #pragma unroll
-                for (int kk = 0; kk < kStageTokens / 16; ++kk)
-                    mma_ts(tmem + 2 * kStageTokens, p_tmem + kk * 8,
-                           smem_desc(vb + kk * 2048, kStageTokens * 128, 1024), kIdescPV,
-                           (next_pv > 0 || kk > 0) ? 1u : 0u);
-                tc_commit(smem_u32(&c.vempty[v_stage]));
-                if (next_pv + 1 == n_pairs) tc_commit(smem_u32(&c.o_full));
+                    for (int kk = 0; kk < kStageTokens / 16; ++kk)
+                        mma_ts(tmem + 2 * kStageTokens, p_tmem + kk * 8, smem_desc_at(vb + kk * (2048 >> 4)), kIdescPV,
+                               (next_pv > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit(smem_u32(&c.vempty[v_stage]));
+                    if (next_pv + 1 == n_pairs) tc_commit(smem_u32(&c.o_full));
+                }
                 if (++v_stage == kStages) {
                     v_stage = 0;
                     v_phase ^= 1;
@@ -2084,18 +2126,17 @@ __device__ void tc_issue(const DecodeArgs& a, CtlTc& c, const uint8_t* ring, con
             if (progress) {
                 spins = 0;
                 idle_since = 0;
-            } else if ((++spins & 1023) == 0) {  // bounded: give up after the wait limit
+            } else if ((++spins & 63) == 0) {  // bounded: give up after the wait limit
                 const uint64_t now = global_ns();
                 if (idle_since == 0) {
                     idle_since = now;
-                } else if (now - idle_since > kWaitLimitNs) {
+                } else if (__any_sync(0xffffffffu, now - idle_since > kWaitLimitNs)) {
                     note_timeout(a, c, 2);
                     return;
                 }
             }
         }
-        gs += n_pairs;
-        mbar_arrive(smem_u32(&c.uempty[q]));
+        if (leader) mbar_arrive(smem_u32(&c.uempty[q]));
     }
 }
 
@@ -2357,7 +2398,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
     } else if (warp == kTcFetcherWarp) {
         tc_fetch<HD, CAP>(a, words, ctl, qbuf);
     } else if (warp == kTcIssuerWarp) {
-        if ((tid & 31) == 0) tc_issue<HD>(a, ctl, ring, qbuf);
+        tc_issue<HD>(a, ctl, ring, qbuf);
     }
     tc_fence_before();
     __syncthreads();
