@@ -267,9 +267,9 @@ tp_status tp_prefill(tp_tree* tree, const tp_node* nodes, const int32_t* n_queri
  * root-to-node paths), the same leaves / nodes / n_queries / flags and the
  * same row layouts, but Q_host, O_host and LSE_host are host memory. The
  * library uploads Q into device staging of its own, runs the attention there
- * and downloads O and LSE (a decode call's kernels may write them to
- * page-locked memory themselves). Library engineering with no counterpart in the
- * paper.
+ * and downloads O and LSE (a decode call's kernels write small results to
+ * page-locked memory themselves). Library engineering with no counterpart in
+ * the paper.
  *
  * Asynchronous, like every attention call: the copies and the kernels are
  * enqueued and the call returns. Q_host must stay unchanged, and O_host /

@@ -740,22 +740,20 @@ void* mapped_host(void* p, uintptr_t align) {
 }
 
 // Whether a decode call's merge writes its results to page-locked host memory
-// itself (each row once, whole lines) instead of leaving them to a download.
-// A caller that waits after each call saves the download and the hop to its
-// stream (256 leaves 149 us a call -> 141, 8 leaves 46 -> 38); back to back,
-// downloads overlap the next call while the merge's stores to the host do not
-// (256 leaves 94 us a call against 102, 1024 leaves 329 / 356, but 16 leaves,
-// 115 KB, 20.2 either way). So: small results always, others when the call
-// before has finished.
+// itself (each row once, whole lines) instead of leaving them to a download: a
+// caller that waits after each call saves the download and the hop to its
+// stream (8 leaves 46 us a call -> 37; a burst of 16 leaves' calls, 115 KB
+// each, 20.2 us a call either way). Small results only: larger ones' stores
+// hold up the next call's attention, which a download does not (256 leaves,
+// 1.8 MB: one call 151 us -> 143 but two 235 -> 248; 1024 leaves, 7.3 MB: one
+// 449 -> 435, two 763 -> 800, twenty 6542 -> 6573 even if only a call that
+// finds the stream idle writes itself).
 constexpr int64_t kDirectBytes = 128 << 10;
 
 bool write_direct(const tp_tree* t, int64_t o_bytes) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(t->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-    if (o_bytes <= kDirectBytes || t->hp_calls == 0) return true;
-    const cudaError_t e = cudaEventQuery(t->hp_done[(t->hp_calls - 1) & 1]);
-    if (e != cudaSuccess) cudaGetLastError();  // (not ready is an error code too)
-    return e == cudaSuccess;
+    return o_bytes <= kDirectBytes && cudaStreamIsCapturing(t->stream, &cap) == cudaSuccess &&
+           cap == cudaStreamCaptureStatusNone;
 }
 
 // One host-buffer call: upload Q into staging slot b once the attention that
@@ -825,9 +823,10 @@ tp_status tp_decode_host(tp_tree* t, const tp_node* leaves, int32_t n, const voi
     if (!t->cfg.pool) return fail(t, TP_ERR_INVALID_ARG, "metadata-only tree cannot decode");
     if (!Q_host || !O_host || !LSE_host) return fail(t, TP_ERR_INVALID_ARG, "Q/O/LSE host pointer is NULL");
     const int64_t row = (int64_t)t->cfg.num_q_heads * t->cfg.head_dim;
-    void* O_dev = mapped_host(O_host, 16);
-    float* LSE_dev = (float*)mapped_host(LSE_host, 4);
-    const bool direct = O_dev && LSE_dev && write_direct(t, n * row * 2);
+    const bool small = write_direct(t, n * row * 2);
+    void* O_dev = small ? mapped_host(O_host, 16) : nullptr;
+    float* LSE_dev = small ? (float*)mapped_host(LSE_host, 4) : nullptr;
+    const bool direct = O_dev && LSE_dev;
     return run_host(t, n * row * 2, direct ? 0 : n * row * 2, direct ? 0 : (int64_t)n * t->cfg.num_q_heads * 4, Q_host,
                     O_host, LSE_host, [&](const void* Q, void* O, float* LSE) {
                         return tp_decode_ex(t, leaves, n, Q, direct ? O_dev : O, direct ? LSE_dev : LSE, flags);
