@@ -738,7 +738,7 @@ def bench_advantage(args):
         "roofline": {"bound": "hbm", "achieved": algo / (ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                      "frac": algo / (ms / 1e3) / 1e9 / peak, "traffic": None,
                      "kernel": "advantage_kernel",
-                     "note": "one cooperative launch (fp64 sub-group sums, pooled A_i, normalisation); a few "
+                     "note": "one launch (fp64 sub-group sums, pooled A_i, normalisation); a few "
                              "hundred KB per call: bound by latency and fp64 arithmetic, not bandwidth",
                      "peak_source": f"{kind} hbm_gbs"},
         "e2e": {"value": len(leaves) / e2e_s, "unit": "trajectories/s", "h2d_bytes_per_step": 8 * len(leaves),
