@@ -790,21 +790,23 @@ tp_status run_host(tp_tree* t, int64_t q_bytes, int64_t o_bytes, int64_t lse_byt
     if (e == cudaSuccess) e = cudaEventRecord(t->hp_up[b], t->hp_h2d);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(t->stream, t->hp_up[b], 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(t->stream, t->hp_down[b], 0);
-    if (e == cudaSuccess && o_bytes == 0)  // nor may an earlier download land after these kernels' results
-        e = cudaStreamWaitEvent(t->stream, t->hp_down[b ^ 1], 0);
+    if (o_bytes == 0) {  // nor may the other slot's download, or its kernels on another stream, land after these results
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(t->stream, t->hp_down[b ^ 1], 0);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(t->stream, t->hp_done[b ^ 1], 0);
+    }
     if (e != cudaSuccess) return cuda_fail(t, e, "query upload");
     st = run(t->hp_q[b], t->hp_o[b], (float*)t->hp_lse[b]);
     if (st != TP_OK) return st;
+    // The download stream takes part either way: what waits for it (tp_sync, a
+    // growing slot, tp_tree_destroy) covers results that the kernels wrote, also
+    // when the tree has been given another stream since.
     e = cudaEventRecord(t->hp_done[b], t->stream);
-    if (o_bytes == 0) {
-        if (e != cudaSuccess) return cuda_fail(t, e, "cudaEventRecord");
-        ++t->hp_calls;
-        return TP_OK;
-    }
     if (e == cudaSuccess) e = cudaStreamWaitEvent(t->hp_d2h, t->hp_done[b], 0);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(Oh, t->hp_o[b], (size_t)o_bytes, cudaMemcpyDeviceToHost, t->hp_d2h);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(Lh, t->hp_lse[b], (size_t)lse_bytes, cudaMemcpyDeviceToHost, t->hp_d2h);
-    if (e == cudaSuccess) e = cudaEventRecord(t->hp_down[b], t->hp_d2h);
+    if (o_bytes > 0) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(Oh, t->hp_o[b], (size_t)o_bytes, cudaMemcpyDeviceToHost, t->hp_d2h);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(Lh, t->hp_lse[b], (size_t)lse_bytes, cudaMemcpyDeviceToHost, t->hp_d2h);
+        if (e == cudaSuccess) e = cudaEventRecord(t->hp_down[b], t->hp_d2h);
+    }
     if (e != cudaSuccess) return cuda_fail(t, e, "result download");
     ++t->hp_calls;
     return TP_OK;

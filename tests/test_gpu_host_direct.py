@@ -2,7 +2,8 @@
 itself, or leaves to a download: bit-identical to the device-buffer call in
 either case -- waiting after each call, back to back, small and large results,
 one pinned and one pageable buffer, buffers at odd offsets, and the same pinned
-buffers as before a call with others."""
+buffers as before a call with others; and tp_sync covers them after the tree
+has been given another stream."""
 import pytest
 import torch
 
@@ -57,4 +58,41 @@ def test_results_written_to_the_host(prompts):
             tp.tp_decode_host(f.handle, leaves, pinned[k], O, lse)
         f.sync()
         assert torch.equal(O, want[3][0]) and torch.equal(lse_pinned, want[3][1]) and torch.equal(lse_plain, want[2][1])
+    f.close()
+
+
+# the kernels of the call sit behind ~50 ms of other work on the stream that the tree had then
+@pytest.mark.parametrize("n", [1, 8])
+def test_sync_after_the_stream_changed(n):
+    script = workloads.no_sharing(seed=4, n_seqs=n, segments=1)
+    f, ids = build_forest(script)
+    h, leaves = script.heads, [ids[x] for x in script.leaves]
+    Q = script.q(DEV)
+    O_ref, LSE_ref = f.decode(leaves, Q, flags=tp.TP_MMA_SYNC)
+    f.sync()
+    want = O_ref.cpu(), LSE_ref.cpu()
+    Qh = Q.cpu().pin_memory()
+    old, new = torch.cuda.Stream(), torch.cuda.Stream()
+    tp.tp_set_stream(f.handle, old.cuda_stream)
+    outs = [(torch.zeros((n, h.num_q_heads, h.head_dim), dtype=torch.bfloat16).pin_memory(),
+             torch.zeros((n, h.num_q_heads)).pin_memory()) for _ in range(3)]
+    tp.tp_decode_host(f.handle, leaves, Qh, *outs[0], tp.TP_MMA_SYNC)  # first buffers made, everything idle
+    f.sync()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(old):
+        torch.cuda._sleep(100_000_000)
+    tp.tp_decode_host(f.handle, leaves, Qh, *outs[1], tp.TP_MMA_SYNC)
+    tp.tp_set_stream(f.handle, new.cuda_stream)
+    f.sync()  # the new stream is idle: the results are still on the old one
+    assert torch.equal(outs[1][0], want[0]) and torch.equal(outs[1][1], want[1])
+    # a call on the new stream into the buffers of one still waiting on the old: the later call's results stay
+    tp.tp_set_stream(f.handle, old.cuda_stream)
+    with torch.cuda.stream(old):
+        torch.cuda._sleep(100_000_000)
+    other = torch.zeros_like(Qh).pin_memory()
+    tp.tp_decode_host(f.handle, leaves, other, *outs[2], tp.TP_MMA_SYNC)
+    tp.tp_set_stream(f.handle, new.cuda_stream)
+    tp.tp_decode_host(f.handle, leaves, Qh, *outs[2], tp.TP_MMA_SYNC)
+    f.sync()
+    assert torch.equal(outs[2][0], want[0]) and torch.equal(outs[2][1], want[1])
     f.close()
