@@ -2020,13 +2020,15 @@ __device__ __forceinline__ bool elect_one() {
     return e != 0;
 }
 
-// mbar_test and mbar_try_wait with a warp-uniform answer
+// mbar_test and mbar_try_wait with a warp-uniform answer: yes once every lane
+// has seen the phase itself, the one that issues among them (a vote orders no
+// memory, so another lane's observation would not cover what it reads).
 __device__ __forceinline__ bool warp_test(uint32_t bar, uint32_t parity) {
-    return __any_sync(0xffffffffu, mbar_test(bar, parity));
+    return __all_sync(0xffffffffu, mbar_test(bar, parity));
 }
 
 __device__ __forceinline__ bool warp_try_wait(uint32_t bar, uint32_t parity) {
-    return __any_sync(0xffffffffu, mbar_try_wait(bar, parity));
+    return __all_sync(0xffffffffu, mbar_try_wait(bar, parity));
 }
 
 // MMA issuer warp: every lane runs the event loop, one elected lane issues.

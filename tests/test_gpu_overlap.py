@@ -1,7 +1,8 @@
 """Kernels that start while their predecessor still runs: calls back to back
 without waiting give the results of the same calls run one at a time -- two
 trees on one stream, appends between decodes, every routing (tcgen05 units
-first, last, none), prefill between decodes, and a replayed CUDA graph."""
+first, last, none), prefill between decodes, a replayed CUDA graph, and the
+tcgen05 units' results over many repeats of a call."""
 import pytest
 import torch
 
@@ -104,4 +105,22 @@ def test_captured_decode_replays():
         for (O, LSE), (O2, LSE2) in zip(want, got):
             assert torch.equal(O, O2) and torch.equal(LSE, LSE2)
     f.sync()
+    f.close()
+
+
+# An operand that the tensor core reads before it has landed shows as a result that differs from one repeat to the next:
+# short units (a few stages each, every one started by the copies' arrival) and long ones, decode and prefill
+@pytest.mark.parametrize("heads", [workloads.Heads(28, 4, 128), workloads.Heads(16, 2, 64)])
+@pytest.mark.parametrize("tokens,queries", [(40, 40), (717, 717), (2000, 130)])
+def test_tcgen05_results_repeat(heads, tokens, queries):
+    s = workloads.single_path(seed=6, lengths=(tokens,), heads=heads)
+    f, ids = build_forest(s)
+    leaf = ids[s.leaves[0]]
+    Q, Qd = s.q(DEV, n=queries), s.q(DEV, n=200)
+    outs = [(f.prefill([leaf], [queries], Q), f.decode([leaf] * 200, Qd, flags=tp.TP_DECODE_ALL_TCGEN05))
+            for _ in range(60)]
+    f.sync()
+    for pre, dec in outs[1:]:
+        for a, b in zip(pre + dec, outs[0][0] + outs[0][1]):
+            assert torch.equal(a, b)
     f.close()
