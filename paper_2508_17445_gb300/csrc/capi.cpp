@@ -5,6 +5,7 @@
 #include <new>
 #include <string>
 
+#include <cuda.h>
 #include <nvtx3/nvToolsExt.h>
 
 #include "forest.h"
@@ -728,15 +729,33 @@ tp_status tp_prefill(tp_tree* t, const tp_node* nodes, const int32_t* n_queries,
 }  // extern "C"
 
 namespace {
-// Device address of page-locked host memory, null for any other.
-void* mapped_host(void* p, uintptr_t align) {
-    cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return at.type == cudaMemoryTypeHost && at.devicePointer && aligned(at.devicePointer, align) ? at.devicePointer
-                                                                                                 : nullptr;
+// The driver's range query (the runtime's pointer attributes have no extent).
+decltype(&cuPointerGetAttributes) pointer_query() {
+    static const auto fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &found) != cudaSuccess)
+            cudaGetLastError();
+        return (decltype(&cuPointerGetAttributes))(found == cudaDriverEntryPointSuccess ? f : nullptr);
+    }();
+    return fn;
+}
+
+// Device address of `bytes` bytes of page-locked host memory that kernels may
+// write, null for any other.
+void* mapped_host(void* p, int64_t bytes, uint64_t align) {
+    const auto query = pointer_query();
+    if (!query) return nullptr;
+    unsigned type = 0, managed = 0, access = 0;
+    tp::HostRange r;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE,      CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_POINTER,   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE,       CU_POINTER_ATTRIBUTE_ACCESS_FLAGS};
+    void* into[] = {&type, &managed, &r.device, &r.start, &r.size, &access};
+    if (query(6, what, into, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return nullptr;
+    r.page_locked = type == CU_MEMORYTYPE_HOST && !managed;
+    r.writable = access == CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE;
+    return tp::host_stores_ok(r, (uintptr_t)p, (uint64_t)bytes, align) ? (void*)(uintptr_t)r.device : nullptr;
 }
 
 // Whether a decode call's merge writes its results to page-locked host memory
@@ -826,8 +845,8 @@ tp_status tp_decode_host(tp_tree* t, const tp_node* leaves, int32_t n, const voi
     if (!Q_host || !O_host || !LSE_host) return fail(t, TP_ERR_INVALID_ARG, "Q/O/LSE host pointer is NULL");
     const int64_t row = (int64_t)t->cfg.num_q_heads * t->cfg.head_dim;
     const bool small = write_direct(t, n * row * 2);
-    void* O_dev = small ? mapped_host(O_host, 16) : nullptr;
-    float* LSE_dev = small ? (float*)mapped_host(LSE_host, 4) : nullptr;
+    void* O_dev = small ? mapped_host(O_host, n * row * 2, 16) : nullptr;
+    float* LSE_dev = O_dev ? (float*)mapped_host(LSE_host, (int64_t)n * t->cfg.num_q_heads * 4, 4) : nullptr;
     const bool direct = O_dev && LSE_dev;
     return run_host(t, n * row * 2, direct ? 0 : n * row * 2, direct ? 0 : (int64_t)n * t->cfg.num_q_heads * 4, Q_host,
                     O_host, LSE_host, [&](const void* Q, void* O, float* LSE) {

@@ -119,6 +119,23 @@ TP_HD bool unit_ok(int32_t tile_off, int32_t n_tiles, int32_t occ_off, int32_t r
 // Occurrence `i`'s merge entries [beg, end).
 TP_HD bool merge_range_ok(int32_t beg, int32_t end, int32_t n_merge) { return 0 <= beg && beg <= end && end <= n_merge; }
 
+// ---- results written straight to host memory ------------------------------
+// What the driver says about a host pointer: whether it is page-locked host
+// memory, the address the device reaches it at, the one allocation or
+// registration that holds it, and whether the device may write there.
+struct HostRange {
+    bool page_locked = false, writable = false;
+    uint64_t device = 0, start = 0, size = 0;
+};
+
+// Whether kernels may store `bytes` bytes at host address p: every one of them
+// in that one range (two neighbouring ranges may have a gap between them, so
+// the last byte's answer would not do), reached at an `align`-aligned address.
+inline bool host_stores_ok(const HostRange& r, uint64_t p, uint64_t bytes, uint64_t align) {
+    return r.page_locked && r.writable && r.device != 0 && r.device % align == 0 && r.start <= p &&
+           p - r.start <= r.size && bytes <= r.size - (p - r.start);
+}
+
 // ---- device launch arguments --------------------------------------------
 struct DecodeArgs {
     const int32_t* units;
