@@ -166,9 +166,13 @@ tp_status tp_prune(tp_tree* tree, tp_node leaf);
  * O: device bf16 [n][num_q_heads][head_dim]; LSE: device fp32
  * [n][num_q_heads], natural log. Q, O 16-byte aligned, LSE 4-byte aligned.
  * Each path segment shared by several listed leaves is read from HBM once
- * for all of them. n == 0 is a no-op. Asynchronous on the tree's stream.
+ * for all of them. n == 0 is a no-op. Asynchronous on the tree's stream. A
+ * call that finds its schedule cached (same leaves and flags as the last one,
+ * no change to the tree since) may be captured into a CUDA graph; the graph
+ * may be replayed until the tree changes or other leaves are decoded.
  * Errors: TP_ERR_BAD_NODE, TP_ERR_NOT_LEAF, TP_ERR_EMPTY_PATH,
- * TP_ERR_INVALID_ARG, TP_ERR_OOM / TP_ERR_CUDA (library scratch).
+ * TP_ERR_INVALID_ARG (also for any other call while the stream is being
+ * captured), TP_ERR_OOM / TP_ERR_CUDA (library scratch).
  */
 tp_status tp_decode(tp_tree* tree, const tp_node* leaves, int32_t n, const void* Q, void* O,
                     float* LSE);
@@ -233,7 +237,9 @@ tp_status tp_decode_noalloc(tp_tree* tree, const tp_node* leaves, int32_t n, con
  * blocks reuses its cached schedule (only the leaves' last-block token
  * counts are rewritten on the device). n == 0 is a no-op. Errors:
  * TP_ERR_BAD_NODE, TP_ERR_FROZEN, TP_ERR_OOM (nothing is appended),
- * TP_ERR_INVALID_ARG (also for a node listed twice).
+ * TP_ERR_INVALID_ARG (also for a node listed twice, and, nothing appended,
+ * while the tree's stream is being captured into a CUDA graph: a replay
+ * would write the same pool slots again).
  */
 tp_status tp_append_tokens(tp_tree* tree, const tp_node* nodes, int32_t n, const void* K, const void* V);
 
@@ -257,7 +263,9 @@ tp_status tp_append_tokens(tp_tree* tree, const tp_node* nodes, int32_t n, const
  * units instead. A row block whose path fits one unit writes O and
  * LSE directly; longer ones are split and merged by log-sum-exp.
  * Asynchronous on the tree's stream. Errors: TP_ERR_BAD_NODE,
- * TP_ERR_INVALID_ARG, TP_ERR_OOM / TP_ERR_CUDA (library scratch).
+ * TP_ERR_INVALID_ARG (also while the stream is being captured into a CUDA
+ * graph: the schedule is made anew for each call), TP_ERR_OOM / TP_ERR_CUDA
+ * (library scratch).
  */
 tp_status tp_prefill(tp_tree* tree, const tp_node* nodes, const int32_t* n_queries, int32_t n, const void* Q,
                      void* O, float* LSE, uint32_t flags);

@@ -229,6 +229,19 @@ tp_status ensure_device(tp_tree* t, T*& ptr, int64_t& cap, int64_t need, const c
     return st;
 }
 
+// Refuses a call that carries the tree's state of now (pool slots, tile words)
+// while the stream is being captured: a replay would repeat it, writing slots
+// and reading blocks that have since changed hands, and the tree would count
+// what only a replay does.
+tp_status refuse_capture(tp_tree* t, const char* call) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(t->stream, &cap);
+    if (e != cudaSuccess) return cuda_fail(t, e, "stream capture query");
+    if (cap != cudaStreamCaptureStatusNone)
+        return fail(t, TP_ERR_INVALID_ARG, std::string(call) + " cannot run while its stream is being captured");
+    return TP_OK;
+}
+
 tp_status run_schedule(tp_tree* t, const tp::Schedule& S, const void* Q, void* O, float* LSE,
                        const int32_t* d_sched = nullptr, const tp::StepWords* words = nullptr);
 
@@ -472,7 +485,8 @@ tp_status tp_append_tokens(tp_tree* t, const tp_node* nodes, int32_t n, const vo
         return fail(t, TP_ERR_INVALID_ARG, "metadata-only tree: K and V must be NULL");
     }
     int64_t need = 0;
-    tp_status st = tp::append_tokens_plan(t, nodes, n, &need);
+    tp_status st = t->cfg.pool ? refuse_capture(t, "tp_append_tokens") : TP_OK;
+    if (st == TP_OK) st = tp::append_tokens_plan(t, nodes, n, &need);
     if (st != TP_OK) return st;
     const uint64_t before = t->version;
     tp::append_tokens_commit(t, nodes, n, need);
@@ -640,6 +654,10 @@ tp_status tp_decode_ex(tp_tree* t, const tp_node* leaves, int32_t n, const void*
                            t->sched_leaves.size() == (size_t)n &&
                            std::equal(leaves, leaves + n, t->sched_leaves.begin());
     tp::Schedule& S = t->sched;
+    if (!same_call || t->sched_version != t->version) {  // the device's schedule has to change
+        tp_status st = refuse_capture(t, "a decode call with a new or changed schedule");
+        if (st != TP_OK) return st;
+    }
     if (same_call && t->sched_version != t->version && t->sched_struct == t->struct_version) {
         tp_status st = patch_cached_schedule(t);
         if (st != TP_OK) {
@@ -677,6 +695,8 @@ tp_status tp_prefill(tp_tree* t, const tp_node* nodes, const int32_t* n_queries,
     tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S, true);
     if (st != TP_OK) return st;
     if (S.n == 0) return TP_OK;
+    st = refuse_capture(t, "tp_prefill");
+    if (st != TP_OK) return st;
     // A small schedule without split rows travels with the attention launch:
     // no buffer, copy stream or event (calls back to back: 40 queries 14.5 ->
     // 9.6 us, a 717-token prompt 20.9 -> 16.8).
@@ -982,18 +1002,14 @@ tp_status tp_decode_noalloc(tp_tree* t, const tp_node* leaves, int32_t n, const 
     if (!t->cfg.pool) return fail(t, TP_ERR_INVALID_ARG, "metadata-only tree cannot decode");
     if (!Q || !O || !LSE || !aligned(Q, 16) || !aligned(O, 16) || !aligned(LSE, 4))
         return fail(t, TP_ERR_INVALID_ARG, "Q/O must be 16-byte and LSE 4-byte aligned device pointers");
-    // The schedule is uploaded from a host vector that dies on return: a
-    // captured copy node would read it again on every replay. Refuse capture.
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaError_t ce = cudaStreamIsCapturing(t->stream, &cap);
-    if (ce != cudaSuccess) return cuda_fail(t, ce, "stream capture query");
-    if (cap != cudaStreamCaptureStatusNone)
-        return fail(t, TP_ERR_INVALID_ARG, "tp_decode_noalloc cannot run while its stream is being captured");
+    // (Nor does the host vector that the schedule is uploaded from outlive the call.)
+    tp_status st = refuse_capture(t, "tp_decode_noalloc");
+    if (st != TP_OK) return st;
     tp::Schedule S;  // host-side only; the tree's schedule cache is left alone
     const int32_t hq = t->cfg.num_q_heads, hd = t->cfg.head_dim;
     int64_t sched_bytes = 0, part_bytes = 0;
     for (const bool coarse : {false, true}) {  // the schedule with the fewest partials where the other does not fit
-        tp_status st = tp::build_schedule(t, leaves, n, flags & ~TP_DECODE_NO_CACHE, S, coarse);
+        st = tp::build_schedule(t, leaves, n, flags & ~TP_DECODE_NO_CACHE, S, coarse);
         if (st != TP_OK) return st;
         sched_bytes = ((int64_t)S.words.size() * 4 + 255) / 256 * 256;
         part_bytes = (int64_t)S.n_slots * hq * (hd + 1) * 4;
