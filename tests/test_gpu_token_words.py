@@ -67,23 +67,34 @@ def test_append_to_other_leaves_than_the_cached_ones():
     f.close()
 
 
+# The decode still waits on the old stream while the new one appends: its schedule must not change under it, so the
+# append carries no patch, and the next decode makes up for it.
 def test_stream_changed_between_decode_and_append():
     f, leaves, draw = forest(64, 3)
     Q = draw(64, 2)
-    main, other = torch.cuda.current_stream(), torch.cuda.Stream()
+    streams = torch.cuda.Stream(), torch.cuda.Stream()
+    new = lambda: (torch.empty_like(Q), torch.empty((64, 2), device=DEV))  # noqa: E731
+    tp.tp_set_stream(f.handle, streams[0].cuda_stream)
     for k in range(6):
-        f.decode(leaves, Q)
-        s = (other, main)[k & 1]
-        tp.tp_set_stream(f.handle, s.cuda_stream)
+        old, s = streams[k & 1], streams[~k & 1]
         K, V = draw(64, 1), draw(64, 1)
+        want, got = new(), new()
         torch.cuda.synchronize()
+        f.decode(leaves, Q, out=want)  # caches or patches the schedule for the tokens of now
+        f.sync()
+        with torch.cuda.stream(old):
+            torch.cuda._sleep(20_000_000)
+        f.decode(leaves, Q, out=got)
+        tp.tp_set_stream(f.handle, s.cuda_stream)
         f.append_tokens(leaves, K, V)
-        O, LSE = torch.empty_like(Q), torch.empty((64, 2), device=DEV)
-        f.decode(leaves, Q, out=(O, LSE))
-        O2, LSE2 = torch.empty_like(Q), torch.empty((64, 2), device=DEV)
-        f.decode(leaves, Q, flags=tp.TP_DECODE_NO_CACHE, out=(O2, LSE2))
+        s.wait_stream(old)
+        after, fresh = new(), new()
+        f.decode(leaves, Q, out=after)
+        f.decode(leaves, Q, flags=tp.TP_DECODE_NO_CACHE, out=fresh)
         torch.cuda.synchronize()
-        assert torch.equal(O, O2) and torch.equal(LSE, LSE2)
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+        assert torch.equal(after[0], fresh[0]) and torch.equal(after[1], fresh[1])
+        assert not torch.equal(after[0], want[0])
     f.close()
 
 
