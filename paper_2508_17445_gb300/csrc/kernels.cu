@@ -637,9 +637,11 @@ __global__ void __launch_bounds__(kAdvAbarThreads) advantage_abar_kernel(const A
 //    together;
 //  - a group of one contributes R_i - R_i = 0 and is skipped; other means and
 //    the mean over |J_i| groups are divisions by small integers (div_small);
-//  - sum A_i and sum A_i^2 meet in two atomics per warp. The groups' means are
-//    taken out of A_i already, so their own mean stays below their spread and
-//    E[A^2] - E[A]^2 does not cancel.
+//  - sum A_i and sum A_i^2 meet in two atomics per warp. E[A^2] - E[A]^2 loses
+//    at most a factor N = the accepted outputs to cancellation, N 2^-53 < 5e-12
+//    of the variance here: the A_i weighted by |J_i| sum to zero, so equal A_i
+//    (shallow outputs) need one of the other sign (a deep one, near 0), and the
+//    mean is at most ~sqrt(N) deviations.
 // 1024 trajectories, 10k nodes: four launches 32 us a call, one with plain
 // divisions and two-pass statistics 30.7, this one over a grid 19.2 (three
 // grid barriers of ~1.8 us, the walk 1.8, the means ~2), in one cluster
@@ -757,7 +759,8 @@ __global__ void __launch_bounds__(CLUSTER ? kAdvClusterThreads : kAdvCta)
             const int32_t c = __ldcg(&w.cnt[x]);
             if (c != 1) acc += r - div_small(__ldcg(&w.sum[x]), c);
         }
-        s = div_small(acc, depth);
+        // (an infinite or NaN reward's own groups of one were skipped, not r - r)
+        s = isfinite(rf) ? div_small(acc, depth) : (double)rf - (double)rf;
     }
     if ((int)(threadIdx.x & ~31u) < per_cta) {  // warps that hold outputs
         const int n_warp = __popc(__ballot_sync(0xffffffffu, accepted));
@@ -778,13 +781,13 @@ __global__ void __launch_bounds__(CLUSTER ? kAdvClusterThreads : kAdvCta)
     const int n = __ldcg(&w.flags[1]);
     const double inv_n = n > 0 ? div_small(1.0, n) : 0.0;
     const double mean = __ldcg(&w.tot[0]) * inv_n;
-    const double var = fmax(0.0, fma(-mean, mean, __ldcg(&w.tot[1]) * inv_n));
-    const double inv_sd = var > 0.0 ? rsqrt(var) : 0.0;
-    if (mine) a.adv[i] = accepted ? (float)(s * inv_sd) : 0.f;
+    const double v = fma(-mean, mean, __ldcg(&w.tot[1]) * inv_n), var = v < 0.0 ? 0.0 : v;
+    const double inv_sd = var > 0.0 ? rsqrt(var) : 0.0;  // 0 too where an A_i is not finite and var is NaN
+    if (mine) a.adv[i] = accepted && inv_sd > 0.0 ? (float)(s * inv_sd) : 0.f;
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.stats) {
         a.stats[0] = (double)n;
         a.stats[1] = mean;
-        a.stats[2] = var * inv_sd;
+        a.stats[2] = var > 0.0 ? var * inv_sd : var;
         a.stats[3] = __ldcg(&w.flags[0]) ? 1.0 : 0.0;
     }
 }

@@ -1,13 +1,14 @@
 """The tree advantage over the sizes where its launch changes: one cluster (up
 to 1024 outputs) and a grid, the last output of a CTA, one to four warps of
 outputs per CTA, and more outputs than the grid has threads (then four
-launches); paths deeper than the ancestors a thread keeps. Oracle and tolerance
-of test_gpu_rollout.py (fp64 accumulation, fp32 output: 1e-6 (|adv| + 1))."""
+launches); paths deeper than the ancestors a thread keeps; rewards that
+are not finite. Oracle and tolerance of test_gpu_rollout.py (fp64 accumulation,
+fp32 output: 1e-6 (|adv| + 1))."""
 import numpy as np
 import pytest
 
 from test_gpu_parity import _built  # noqa: F401
-from test_gpu_rollout import check_advantage
+from test_gpu_rollout import check_advantage, run_advantage
 
 pytestmark = pytest.mark.gpu
 
@@ -47,3 +48,37 @@ def test_all_equal_and_negative_rewards():
     check_advantage(parent, leaf, np.full(64, 0.25))
     reward = np.where(np.arange(64) < 16, -3.5, reward - 0.5)  # the first prompt's are all equal
     check_advantage(parent, leaf, reward)
+
+
+# one output of depth 600 among shallow ones whose A_i are all equal: the mean of A_i is ~sqrt(n) times its spread, where
+# one-pass statistics lose most
+@pytest.mark.parametrize("n_out", [1000, 1100, 20000])
+def test_one_deep_output_among_shallow_ones(n_out):
+    parent, leaf = [-1], []
+    for _ in range(n_out - 1):
+        parent.append(0)
+        leaf.append(len(parent) - 1)
+    x = 0
+    for _ in range(600):
+        parent.append(x)
+        x = len(parent) - 1
+    check_advantage(parent, leaf + [x], [0.0] * (n_out - 1) + [1.0])
+
+
+# the four launches' answer, whichever launch a call takes: no advantages once a counted A_i is not finite, the deviation
+# says so, and a query whose rewards are all the same value stays left out
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("n_out", [64, 1100, 38913])
+def test_rewards_that_are_not_finite(n_out, value):
+    parent, leaf, reward = flat_trees(n_out, 16, 4, 2)
+    reward[:16] = value  # the first prompt's are all equal: rejected
+    if not np.isnan(value):
+        check_advantage(parent, leaf, reward)
+    reward[20] = value
+    adv, stats = run_advantage(parent, leaf, reward)
+    assert (adv == 0).all() and np.isnan(stats[2]) and stats[3] == 0
+    # alone in every group of its own: beside an output that ends at the root and forms no group
+    parent, leaf, reward = list(parent) + [-1], list(leaf), list(np.where(np.isfinite(reward), reward, 0.0))
+    parent.append(len(parent) - 1)
+    adv, stats = run_advantage(parent, leaf + [len(parent) - 2, len(parent) - 1], reward + [0.0, value])
+    assert (adv == 0).all() and np.isnan(stats[2])
