@@ -632,9 +632,11 @@ __global__ void __launch_bounds__(kAdvAbarThreads) advantage_abar_kernel(const A
 // thread (launch_advantage). What bounds a call is latency, and above all
 // fp64 arithmetic (a warp instruction takes ~64 cycles of its sub-partition, a
 // division or square root over a thousand):
-//  - each thread walks to the root once, while the tables are cleared, and
-//    keeps its ancestors; their sums, and then every (count, sum), go out
-//    together;
+//  - each thread walks to the root once, clears what it passes and keeps its
+//    ancestors; their sums, and then every (count, sum), go out together.
+//    (Whole tables cleared by these few CTAs: 64 outputs in 1M nodes 46.5 us a
+//    call, 1024 in 4M 162; now 7 and 7.5 whatever the table's size, where the
+//    four launches take 26.7 and 39.)
 //  - a group of one contributes R_i - R_i = 0 and is skipped; other means and
 //    the mean over |J_i| groups are divisions by small integers (div_small);
 //  - sum A_i and sum A_i^2 meet in two atomics per warp. E[A^2] - E[A]^2 loses
@@ -646,9 +648,9 @@ __global__ void __launch_bounds__(kAdvAbarThreads) advantage_abar_kernel(const A
 // divisions and two-pass statistics 30.7, this one over a grid 19.2 (three
 // grid barriers of ~1.8 us, the walk 1.8, the means ~2), in one cluster
 // (CLUSTER: up to 1024 outputs, hardware barriers, a warp of outputs on each
-// sub-partition of eight SMs) 15.4.
+// sub-partition of eight SMs) 15.4, without clearing whole tables 13.2.
 constexpr int kAdvCta = 128;    // outputs a CTA may hold: one for each of its first per_cta threads
-constexpr int kAdvClusterThreads = 512, kAdvClusterCtas = 8;  // (the other threads help to clear the tables)
+constexpr int kAdvClusterCtas = 8;
 constexpr int kAdvChain = 64;   // ancestors kept; deeper ones are walked again
 constexpr int kAdvMaxCtas = 2 * 152;
 constexpr int kInvTable = 256;
@@ -670,9 +672,7 @@ __device__ __forceinline__ double div_small(double x, int n) {
 }
 
 template <bool CLUSTER>
-__global__ void __launch_bounds__(CLUSTER ? kAdvClusterThreads : kAdvCta)
-    advantage_kernel(const AdvantageArgs a, int per_cta) {
-    constexpr int kThreads = CLUSTER ? kAdvClusterThreads : kAdvCta;
+__global__ void __launch_bounds__(kAdvCta) advantage_kernel(const AdvantageArgs a, int per_cta) {
     __shared__ int32_t chain[kAdvChain][kAdvCta];
     auto sync_all = [] {
         if constexpr (CLUSTER)
@@ -685,12 +685,6 @@ __global__ void __launch_bounds__(CLUSTER ? kAdvClusterThreads : kAdvCta)
         dep_wait();
     }
     const AdvWs w = adv_ws(a);
-    for (int64_t x = (int64_t)blockIdx.x * kThreads + threadIdx.x; x < a.n_nodes; x += (int64_t)gridDim.x * kThreads) {
-        w.cnt[x] = 0;
-        w.sum[x] = 0.0;
-        w.kmin[x] = 0xffffffffu;
-        w.kmax[x] = 0u;
-    }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         w.tot[0] = w.tot[1] = 0.0;
         w.flags[0] = w.flags[1] = 0;  // malformed table, accepted outputs
@@ -713,13 +707,17 @@ __global__ void __launch_bounds__(CLUSTER ? kAdvClusterThreads : kAdvCta)
                     break;
                 }
                 if (depth < kAdvChain) chain[depth][threadIdx.x] = x;
+                w.cnt[x] = 0;
+                w.sum[x] = 0.0;
                 root = x;
                 ++depth;
             }
+            w.kmin[root] = 0xffffffffu;
+            w.kmax[root] = 0u;
         }
     }
     const int kept = min(depth, kAdvChain);
-    sync_all();  // tables clear
+    sync_all();  // what the outputs reach is clear
     if (mine) {
         int32_t x = -1;
         for (int k = 0; k < depth; ++k) {
@@ -2860,7 +2858,7 @@ cudaError_t launch_advantage(const AdvantageArgs& a, cudaStream_t s) {
             attr[1].val.programmaticStreamSerializationAllowed = 1;
             cfg.numAttrs = 2;
             cfg.gridDim = dim3(kAdvClusterCtas);
-            cfg.blockDim = dim3(kAdvClusterThreads);
+            cfg.blockDim = dim3(kAdvCta);
             return cudaLaunchKernelEx(&cfg, advantage_kernel<true>, a, per_cta);
         }
         attr[0].id = cudaLaunchAttributeCooperative;

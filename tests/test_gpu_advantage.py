@@ -1,12 +1,15 @@
 """The tree advantage over the sizes where its launch changes: one cluster (up
 to 1024 outputs) and a grid, the last output of a CTA, one to four warps of
 outputs per CTA, and more outputs than the grid has threads (then four
-launches); paths deeper than the ancestors a thread keeps; rewards that
-are not finite. Oracle and tolerance of test_gpu_rollout.py (fp64 accumulation,
-fp32 output: 1e-6 (|adv| + 1))."""
+launches); paths deeper than the ancestors a thread keeps; node tables far
+larger than what the outputs reach; rewards that are not finite. Oracle and
+tolerance of test_gpu_rollout.py (fp64 accumulation, fp32 output: 1e-6
+(|adv| + 1))."""
 import numpy as np
 import pytest
+import torch
 
+import paper_2508_17445_gb300 as tp
 from test_gpu_parity import _built  # noqa: F401
 from test_gpu_rollout import check_advantage, run_advantage
 
@@ -82,3 +85,24 @@ def test_rewards_that_are_not_finite(n_out, value):
     parent.append(len(parent) - 1)
     adv, stats = run_advantage(parent, leaf + [len(parent) - 2, len(parent) - 1], reward + [0.0, value])
     assert (adv == 0).all() and np.isnan(stats[2])
+
+
+# the outputs reach a small part of the table, and the workspace holds another call's remains
+@pytest.mark.parametrize("n_out", [1, 40, 1024, 1025, 9000])
+def test_large_node_table(n_out):
+    rng = np.random.default_rng(n_out)
+    parent, leaf, reward = flat_trees(n_out, 16, 5, n_out)
+    n_nodes = 300_000
+    ids = rng.permutation(n_nodes)[:len(parent)].astype(np.int32)
+    table = np.full(n_nodes, -1, np.int32)
+    table[ids] = np.where(parent < 0, -1, ids[parent])
+    want = check_advantage(table, ids[leaf], reward)
+    P, L = torch.from_numpy(table).cuda(), torch.from_numpy(ids[leaf]).cuda()
+    R = torch.tensor(reward, dtype=torch.float32, device="cuda:0")
+    ws = torch.full((tp.tp_advantage_workspace_bytes(n_nodes, n_out),), 255, dtype=torch.uint8, device="cuda:0")
+    adv, stats = torch.zeros(n_out, device="cuda:0"), torch.zeros(4, dtype=torch.float64, device="cuda:0")
+    for _ in range(2):
+        tp.tp_tree_advantage(P, L, R, adv, stats, ws)
+        torch.cuda.synchronize()
+        # the sums' order differs from call to call: fp64 rounding
+        assert np.abs(adv.cpu().numpy() - want).max() <= 1e-6
