@@ -261,7 +261,10 @@ tp_status tp_append_tokens(tp_tree* tree, const tp_node* nodes, int32_t n, const
  * <= 64. The work runs as tcgen05 units of up to 128 query rows (whole GQA
  * groups); flags = TP_MMA_SYNC runs it on the mma.sync path in 64-row
  * units instead. A row block whose path fits one unit writes O and
- * LSE directly; longer ones are split and merged by log-sum-exp.
+ * LSE directly; longer ones, and in calls that would end on a few of them
+ * also shorter ones, are split and merged by log-sum-exp. Probabilities enter
+ * P.V in bf16, in calls of few units (up to a few thousand query tokens) as the
+ * sum of two bf16 values.
  * Asynchronous on the tree's stream. Errors: TP_ERR_BAD_NODE,
  * TP_ERR_INVALID_ARG (also while the stream is being captured into a CUDA
  * graph: the schedule is made anew for each call), TP_ERR_OOM / TP_ERR_CUDA

@@ -930,6 +930,7 @@ tp_status run_schedule(tp_tree* t, const tp::Schedule& S, const void* Q, void* O
     if (S.prefill) {
         a.unit_pos = d_sched + S.off_unit_pos;
         a.prefill = 1;
+        a.two_terms = S.two_terms ? 1 : 0;
         a.unit_vis = d_sched + S.off_unit_vis;
         a.w_units = (int32_t)S.off_units;
         a.w_tiles = (int32_t)S.off_tiles;

@@ -516,6 +516,16 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     const int64_t share = std::max<int64_t>(kPrefillMinChunk, (work + kResidentCtas - 1) / kResidentCtas);
     const int32_t chunk =
         (int32_t)std::min<int64_t>(kMaxUnitTiles, longest > share + kPrefillMergeTiles ? share : kMaxUnitTiles);
+    // Calls of fewer than kTargetUnits units of the longest block's length:
+    // P in two bf16 terms. One term leaves 2^-8 of each probability except the
+    // largest of a row's part, so rows kept whole are off by more than rows cut
+    // into parts of kTargetUnits a call (40 queries on 2k tokens: O off by
+    // 0.00234 relative to fp64, cut into 4-tile parts 0.00222, with two terms
+    // 0.00166, its own rounding). The second P.V costs 0-20% of such a call
+    // (717 tokens 13.5 -> 15.4 us, 1.1k 19.5 -> 22.7; as 4-tile parts 53) and
+    // would cost the tensor-bound calls past the line as much, whose rows no
+    // rule would cut.
+    S.two_terms = work < longest * kTargetUnits;
     // 3. units longest first (stable): their number per length, then each
     //    block's units straight to their places in the schedule (with records
     //    built, sorted and split, ragged calls waited for the host: 2160 units

@@ -147,6 +147,7 @@ struct DecodeArgs {
     float* part_lse;    // [slot][Hq], log2-domain partial LSE
     int32_t* err;
     int32_t prefill = 0;
+    int32_t two_terms = 0;  // prefill: P enters P.V as two bf16 terms (see Schedule::two_terms)
     const int32_t* unit_pos = nullptr;  // prefill: path position of each unit's first token
     const int32_t* unit_vis = nullptr;  // prefill: path tokens the unit's first query token sees (each next one: one more)
     // a schedule that travels with the launch (StepWords): its sections' first words
@@ -345,6 +346,8 @@ struct Schedule {
     int32_t n_units = 0, n_tiles = 0, n_occ = 0, n = 0, n_slots = 0, n_merge = 0, n_tensor = 0, n_tc = 0;
     int64_t off_units = 0, off_tiles = 0, off_occ = 0, off_merge_off = 0, off_merge_slot = 0;
     bool prefill = false;
+    // Prefill calls of few units (the rule is in build_prefill_schedule): P in two bf16 terms.
+    bool two_terms = false;
     bool kv_read_once = false;  // see DecodeArgs::kv_read_once
     int64_t off_unit_pos = 0, off_vis = 0, off_unit_vis = 0, off_merge_rec = 0;
     // (leaf node, word index of the last tile of that leaf) for every place a

@@ -211,6 +211,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// Second terms of two probabilities: what their bf16 roundings (a pair, as
+// packed) leave out, in bf16 again.
+__device__ __forceinline__ uint32_t second_terms(float p0, float p1, uint32_t first) {
+    return pack_bf16(p0 - __uint_as_float(first << 16), p1 - __uint_as_float(first & 0xffff0000u));
+}
+
 // 32-byte global store (sm_100 and later); dst must be 32-byte aligned
 __device__ __forceinline__ void st_global_v8(void* dst, const uint32_t* w) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]),
@@ -1348,7 +1354,7 @@ struct TensorPath {
                         l_run[h] *= alpha[h];
                     }
                     // A fragment of P: (row g, tok 2c..) (row g+8, tok 2c..) (row g, tok 2c+8..) (row g+8, ..)
-                    uint32_t pa[4];
+                    uint32_t pa[4], pb[4];  // pb: second terms (CAUSAL, two_terms)
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const float p0 = fast_exp2(s[j][0] - m_use[0]), p1 = fast_exp2(s[j][1] - m_use[0]);
@@ -1357,6 +1363,10 @@ struct TensorPath {
                         l_run[1] += p2 + p3;
                         pa[2 * j] = pack_bf16(p0, p1);
                         pa[2 * j + 1] = pack_bf16(p2, p3);
+                        if constexpr (CAUSAL) {
+                            pb[2 * j] = second_terms(p0, p1, pa[2 * j]);
+                            pb[2 * j + 1] = second_terms(p2, p3, pa[2 * j + 1]);
+                        }
                     }
 #pragma unroll
                     for (int j = 0; j < NT; ++j) {
@@ -1374,6 +1384,10 @@ struct TensorPath {
                         ldsm_x4_t(sv + kv_off<kStageTokens>(tok, ch), b0, b1, b2, b3);
                         mma_bf16(o[2 * dp], pa, b0, b1);
                         mma_bf16(o[2 * dp + 1], pa, b2, b3);
+                        if (CAUSAL && a.two_terms) {
+                            mma_bf16(o[2 * dp], pb, b0, b1);
+                            mma_bf16(o[2 * dp + 1], pb, b2, b3);
+                        }
                     }
                 }
             }
@@ -1790,7 +1804,7 @@ __device__ __forceinline__ void tmem_ld32_nowait(uint32_t taddr, uint32_t (&r)[3
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_st32_nowait(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
         "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
@@ -1799,7 +1813,13 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
         "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
         "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
         : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+    tmem_st32_nowait(taddr, r);
+    tmem_wait_st();
 }
 
 __device__ __forceinline__ UnitDesc read_desc(const int* slot) {
@@ -2040,7 +2060,7 @@ __device__ __forceinline__ bool warp_try_wait(uint32_t bar, uint32_t parity) {
 // one lane that built each descriptor from its address: prefill of 64 prompts
 // 267 -> 251 us, at head_dim 64 1797 -> 1570, 512 segments 4290 -> 4080 (under
 // the power cap), decode over a 2k prefix 305.1 -> 303.7.
-template <int HD>
+template <int HD, bool TWO>
 __device__ void tc_issue(const DecodeArgs& a, CtlTc& c, const uint8_t* ring, const uint8_t* qbuf) {
     constexpr uint32_t kIdescS = mma_idesc<kStageTokens, false>();
     constexpr uint32_t kIdescPV = mma_idesc<HD, true>();
@@ -2113,8 +2133,9 @@ __device__ void tc_issue(const DecodeArgs& a, CtlTc& c, const uint8_t* ring, con
                 const uint32_t p_tmem = tmem + v_stage * kStageTokens;
                 if (leader) {
 #pragma unroll
-                    for (int kk = 0; kk < kStageTokens / 16; ++kk)
-                        mma_ts(tmem + 2 * kStageTokens, p_tmem + kk * 8, smem_desc_at(vb + kk * (2048 >> 4)), kIdescPV,
+                    for (int kk = 0; kk < (TWO ? 2 : 1) * kStageTokens / 16; ++kk)  // second terms after the first
+                        mma_ts(tmem + 2 * kStageTokens, p_tmem + kk * 8,
+                               smem_desc_at(vb + kk % (kStageTokens / 16) * (2048 >> 4)), kIdescPV,
                                (next_pv > 0 || kk > 0) ? 1u : 0u);
                     tc_commit(smem_u32(&c.vempty[v_stage]));
                     if (next_pv + 1 == n_pairs) tc_commit(smem_u32(&c.o_full));
@@ -2144,8 +2165,9 @@ __device__ void tc_issue(const DecodeArgs& a, CtlTc& c, const uint8_t* ring, con
 }
 
 // Softmax + epilogue warps: thread = query row (warp * 32 + lane). CAUSAL
-// (prefill): the row sees only the first vis tokens of its path.
-template <int HD, bool CAUSAL>
+// (prefill): the row sees only the first vis tokens of its path. TWO: P in two
+// terms, the second over the other half of the S columns.
+template <int HD, bool CAUSAL, bool TWO>
 __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int row = warp * 32 + lane;
@@ -2247,7 +2269,7 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
             // P = exp2(s * scale - m_used) as bf16 pairs over the S columns: two
             // scores scaled and shifted per instruction, two pair sums (a row
             // that has seen nothing yet shifts by 0: exp2(-inf) = 0)
-            uint32_t pw[32];
+            uint32_t pw[32], pl[TWO ? 32 : 1];
             float sum;
             {
                 const float sc = a.qk_scale_log2, neg_m = m_used == -INFINITY ? 0.f : -m_used;
@@ -2263,6 +2285,7 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
                         const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
                         acc[(t >> 1) & 1] = f2_add(acc[(t >> 1) & 1], f2_pack(p0, p1));
                         pw[h * 16 + t / 2] = pack_bf16(p0, p1);
+                        if constexpr (TWO) pl[h * 16 + t / 2] = second_terms(p0, p1, pw[h * 16 + t / 2]);
                     }
                 float s0, s1, s2, s3;
                 f2_unpack(acc[0], s0, s1);
@@ -2270,7 +2293,9 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
                 sum = (s0 + s2) + (s1 + s3);
             }
             l += sum;
-            tmem_st32(s_addr, pw);
+            tmem_st32_nowait(s_addr, pw);
+            if constexpr (TWO) tmem_st32_nowait(s_addr + 32, pl);
+            tmem_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&c.p_full[sb]));
@@ -2350,7 +2375,7 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
     }
 }
 
-template <int HD, bool CAUSAL, int CAP>
+template <int HD, bool CAUSAL, bool TWO, int CAP>
 __global__ void __launch_bounds__(kTcThreads, 2)
     decode_tc_kernel(const DecodeArgs a, const __grid_constant__ ParamWords<CAP> words) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -2395,13 +2420,13 @@ __global__ void __launch_bounds__(kTcThreads, 2)
     if (!a.late_wait) dep_wait();
     dep_trigger();
     if (warp < kTcConsumerWarps)
-        tc_consume<HD, CAUSAL>(a, ctl);
+        tc_consume<HD, CAUSAL, TWO>(a, ctl);
     else if (warp == kTcStreamerWarp) {
         if ((tid & 31) == 0) tc_stream<HD>(a, ctl, ring);
     } else if (warp == kTcFetcherWarp) {
         tc_fetch<HD, CAP>(a, words, ctl, qbuf);
     } else if (warp == kTcIssuerWarp) {
-        tc_issue<HD>(a, ctl, ring, qbuf);
+        tc_issue<HD, TWO>(a, ctl, ring, qbuf);
     }
     tc_fence_before();
     __syncthreads();
@@ -2657,16 +2682,16 @@ cudaError_t launch_range(DecodeArgs a, int begin, int end, int32_t* counter, cud
                             decode_smem<HD, KIND>(), s, a);
 }
 
-template <int HD, bool CAUSAL, int CAP>
+template <int HD, bool CAUSAL, bool TWO, int CAP>
 int decode_tc_grid() {
     static int grid = [] {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaFuncSetAttribute(decode_tc_kernel<HD, CAUSAL, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(decode_tc_kernel<HD, CAUSAL, TWO, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  TcSmem<HD>::kBytes) != cudaSuccess)
             return 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_tc_kernel<HD, CAUSAL, CAP>, kTcThreads,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_tc_kernel<HD, CAUSAL, TWO, CAP>, kTcThreads,
                                                           TcSmem<HD>::kBytes) != cudaSuccess)
             return 0;
         // The occupancy query answers 1 for this kernel on GB300 although its
@@ -2676,7 +2701,7 @@ int decode_tc_grid() {
         // unit counter exhausted and exits.
         cudaFuncAttributes fa{};
         int smem_sm = 0, reserved = 0;
-        if (cudaFuncGetAttributes(&fa, decode_tc_kernel<HD, CAUSAL, CAP>) != cudaSuccess) return 0;
+        if (cudaFuncGetAttributes(&fa, decode_tc_kernel<HD, CAUSAL, TWO, CAP>) != cudaSuccess) return 0;
         cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
         const int by_smem = smem_sm / (int)(TcSmem<HD>::kBytes + fa.sharedSizeBytes + reserved);
@@ -2688,11 +2713,11 @@ int decode_tc_grid() {
     return grid;
 }
 
-template <int HD, bool CAUSAL, int CAP>
+template <int HD, bool CAUSAL, bool TWO, int CAP>
 cudaError_t launch_tc_kernel(const DecodeArgs& a, int n_units, cudaStream_t s, const ParamWords<CAP>& words) {
-    const int slots = decode_tc_grid<HD, CAUSAL, CAP>();
+    const int slots = decode_tc_grid<HD, CAUSAL, TWO, CAP>();
     if (slots == 0) return cudaErrorInvalidConfiguration;
-    return launch_dependent(decode_tc_kernel<HD, CAUSAL, CAP>, std::min(n_units, slots), kTcThreads, TcSmem<HD>::kBytes,
+    return launch_dependent(decode_tc_kernel<HD, CAUSAL, TWO, CAP>, std::min(n_units, slots), kTcThreads, TcSmem<HD>::kBytes,
                             s, a, words);
 }
 
@@ -2703,12 +2728,14 @@ cudaError_t launch_tc_range(DecodeArgs a, int begin, int end, int32_t* counter, 
     a.unit_begin = begin;
     a.unit_end = end;
     a.counter = counter;
-    if (words)  // prefill
+    const ParamWords<1> none{};
+    if (words)  // prefill; schedules this small always have P in two terms
         return with_words(*words, [&](const auto& p, const int32_t*) {
-            return launch_tc_kernel<HD, true>(a, end - begin, s, p);
+            return launch_tc_kernel<HD, true, true>(a, end - begin, s, p);
         });
-    return a.prefill ? launch_tc_kernel<HD, true>(a, end - begin, s, ParamWords<1>{})
-                     : launch_tc_kernel<HD, false>(a, end - begin, s, ParamWords<1>{});
+    if (!a.prefill) return launch_tc_kernel<HD, false, false>(a, end - begin, s, none);
+    return a.two_terms ? launch_tc_kernel<HD, true, true>(a, end - begin, s, none)
+                       : launch_tc_kernel<HD, true, false>(a, end - begin, s, none);
 }
 
 // Both attention kernels of a call run side by side: the second is launched

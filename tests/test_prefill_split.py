@@ -1,7 +1,8 @@
 """Where prefill row blocks are split: schedules on both sides of the rule's
 edges cover every visible token once (CPU), and the kernels, which derive each
 row's occurrence and visible length from its unit, agree with the oracle on
-split and unsplit blocks of both head sizes (GPU)."""
+split and unsplit blocks of both head sizes, to O's own rounding where a call's
+probabilities are held in two terms (GPU)."""
 import numpy as np
 import pytest
 
@@ -101,4 +102,35 @@ def test_masked_last_stages(tokens, heads):
     d_o = np.abs(O.float().cpu().numpy().astype(np.float64) - o_ref)
     assert (d_o <= 2.0 ** -8 * (np.abs(o_ref) + a_ref) + 1e-5).all()
     assert np.abs(LSE.cpu().numpy().astype(np.float64) - lse_ref).max() <= 5e-5
+    f.close()
+
+
+# Calls of few units hold each probability in two bf16 terms, split rows or not: what they leave out is 2^-16 of the
+# probability, so O is off by its own rounding (half a unit in the last of its 8 places) and, with what fp32 sums and exp2
+# add to the scores and the sums, 2^-15 of A = sum p |v|. (One bf16 term leaves out up to 2^-8 of each probability, in sum
+# ~2^-13 A over some hundred tokens.)
+# Schedules of both parameter sizes, uploaded, and with split rows
+@pytest.mark.gpu
+@pytest.mark.parametrize("flags", [0, tp.TP_MMA_SYNC])
+@pytest.mark.parametrize("heads", [workloads.Heads(28, 4, 128), workloads.Heads(16, 2, 64)])
+@pytest.mark.parametrize("tokens,queries", [(33, 33), (100, 100), (717, 717), (2000, 2000), (1000, 1), (2100, 40), (9000, 40)])
+def test_probabilities_in_two_terms(tokens, queries, heads, flags):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from test_gpu_parity import _kv_source, build_forest
+    s = workloads.single_path(seed=60 + tokens, lengths=(tokens,), heads=heads)
+    f, ids = build_forest(s)
+    Q = s.q("cuda:0", n=queries)
+    O, LSE = f.prefill([ids[s.leaves[0]]], [queries], Q, flags)
+    f.sync()
+    rows = sorted({0, queries // 3, queries - 1} | set(range(0, queries, 131)))
+    src = _kv_source(s)
+    model = oracle.OracleForest(block_tokens=32, pool_blocks=f.cfg.pool_blocks).replay(s)
+    o_ref, lse_ref = (x[rows] for x in model.prefill([s.leaves[0]], [queries], Q.cpu(), src, indices=rows))
+    abs_src = lambda i: (src(i)[0], oracle.bf16_bits(src(i)[1]) & np.uint16(0x7FFF))  # noqa: E731
+    a_ref = model.prefill([s.leaves[0]], [queries], Q.cpu(), abs_src, indices=rows)[0][rows]
+    d_o = np.abs(O[rows].float().cpu().numpy().astype(np.float64) - o_ref)
+    assert (d_o <= 2.0 ** (np.floor(np.log2(np.abs(o_ref))) - 8) + 2.0 ** -15 * a_ref).all()
+    assert np.abs(LSE[rows].cpu().numpy().astype(np.float64) - lse_ref).max() <= 5e-5
     f.close()
