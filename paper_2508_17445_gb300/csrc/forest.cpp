@@ -110,15 +110,20 @@ constexpr int64_t kFillUnits = kResidentCtas * 2;
 constexpr int64_t kShortUnit = 8;
 constexpr int32_t kMinChunkTiles = 4;
 constexpr int32_t kMaxChunkTiles = 64;
-// Prefill row blocks: the shortest chunk worth a unit, and how many tiles the
-// longest block may have beyond an even share of the work before blocks are
-// split at all. The partials, the merge and its lists cost a call more than
-// the tail they save: split past 16 tiles against 64, a prompt of 1.1k tokens
-// took 41.5 us against 25.3, of 1.4k 48.7 / 31.2, of 1.8k 59 / 41.5; a few
-// queries on a long path are split either way (one on 30k tokens 66.6 us
-// with 1824 units as the target -> 25.0 with these).
-constexpr int64_t kPrefillMinChunk = 8;
-constexpr int64_t kPrefillMergeTiles = 64;
+// Prefill row blocks: the shortest chunk worth a unit, and what splitting
+// blocks costs a call, in tiles of a unit's chain (~0.35 us each on tcgen05,
+// about three times that in the mma.sync units): the merge with its launch and
+// lists, and `tile_bytes` of partials written and read back per tile. Measured
+// against the blocks left whole (tcgen05): one query on 2k tokens 14.2 us
+// against 27, 40 on 2k 17 / 29.5, 32 on eight paths of 2k 19.5 / 27.7, even at
+// 1k (16 / 16); whole prompts with their many partials lose: of 1.1k tokens
+// 41.5 / 25.3 (split past 16 tiles whatever the rows), of 1.8k at head_dim 64
+// 36.4 / 24.1. On mma.sync: 8 queries on 512 tokens 16.3 / 26.9, on 2k 16.5 /
+// 71.7; a prompt of 717 tokens left whole 43.5 against 50 in 4-tile parts.
+struct PrefillCost {
+    int64_t min_chunk, merge_tiles, tile_bytes;
+};
+constexpr PrefillCost kPrefillTc{8, 20, 3 << 19}, kPrefillMma{4, 4, 9 << 19};
 
 // Stable reorder of unit records longest first (a counting sort: n_tiles <=
 // kMaxUnitTiles).
@@ -510,12 +515,22 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     }
     X.node_tile_off[(size_t)n] = (int32_t)X.tiles.size();
     // 2. Row blocks are cut into chunks only where the call would otherwise
-    //    end on a few long ones: the longest block against an even share of
-    //    the work per resident CTA, with kPrefillMergeTiles for what the
-    //    partials and the merge cost.
-    const int64_t share = std::max<int64_t>(kPrefillMinChunk, (work + kResidentCtas - 1) / kResidentCtas);
-    const int32_t chunk =
-        (int32_t)std::min<int64_t>(kMaxUnitTiles, longest > share + kPrefillMergeTiles ? share : kMaxUnitTiles);
+    //    end on a few long ones: the longest block against what the call ends
+    //    on when cut (an even share of the work per resident CTA, or twice
+    //    that where the units no longer run all at once) and the split's cost.
+    const PrefillCost& cost = use_tc ? kPrefillTc : kPrefillMma;
+    const int64_t share = std::max<int64_t>(cost.min_chunk, (work + kResidentCtas - 1) / kResidentCtas);
+    const int64_t cut = (share > cost.min_chunk ? 2 * share : share) + cost.merge_tiles;
+    int64_t slots = 0;
+    if (longest > cut) {
+        size_t k = 0;
+        for (int32_t i = 0; i < n; ++i)
+            for (int32_t o0 = 0; o0 < m[i]; o0 += occ_per_block, ++k)
+                if (X.block_tiles[k] > share)
+                    slots += (X.block_tiles[k] + share - 1) / share * std::min(occ_per_block, m[i] - o0);
+    }
+    const bool split = longest > cut + slots * hq * t->cfg.head_dim * 8 / cost.tile_bytes;
+    const int32_t chunk = (int32_t)std::min<int64_t>(kMaxUnitTiles, split ? share : kMaxUnitTiles);
     // Calls of fewer than kTargetUnits units of the longest block's length:
     // P in two bf16 terms. One term leaves 2^-8 of each probability except the
     // largest of a row's part, so rows kept whole are off by more than rows cut

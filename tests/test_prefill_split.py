@@ -11,25 +11,44 @@ import paper_2508_17445_gb300 as tp
 import workloads
 from test_prefill_host import check_prefill_coverage, metadata_forest
 
-# one row block (18 queries of a 7-row group at most): split past 8 + 64 tiles
-EDGES = [(72 * 32, 1), (72 * 32 + 1, 1), (73 * 32, 18), (128 * 32 + 1, 5), (40 * 32, 40), (9000, 40)]
+# one row block (18 queries of a 7-row group at most) on either side of the lengths that are split: 8 + 20 tiles on
+# tcgen05 and 4 + 4 on mma.sync, a little longer with more rows
+EDGES = [(8 * 32, 1, False, False), (8 * 32 + 1, 1, False, True), (28 * 32, 1, False, True), (28 * 32 + 1, 1, True, True),
+         (28 * 32 + 1, 18, False, True), (30 * 32, 40, False, True), (31 * 32, 40, True, True), (72 * 32, 1, True, True),
+         (72 * 32 + 1, 1, True, True), (73 * 32, 18, True, True), (128 * 32 + 1, 5, True, True), (40 * 32, 40, True, True),
+         (9000, 40, True, True)]
 
 
 @pytest.mark.parametrize("flags", [0, tp.TP_MMA_SYNC])
-@pytest.mark.parametrize("tokens,queries", EDGES)
-def test_split_edges(tokens, queries, flags):
+@pytest.mark.parametrize("tokens,queries,split,split_mma", EDGES)
+def test_split_edges(tokens, queries, split, split_mma, flags):
     s = workloads.single_path(seed=1, lengths=(tokens,), heads=workloads.Heads(28, 4, 128))
     f, ids = metadata_forest(s)
     model = oracle.OracleForest(block_tokens=32, pool_blocks=1 << 10).replay(s)
     check_prefill_coverage(f, model, ids, [s.leaves[0]], [queries], flags)
     d = tp.tp_debug_prefill_schedule(f.handle, [ids[s.leaves[0]]], [queries], flags)
-    assert (d["n_slots"] > 0) == (-(-tokens // 32) > 72)
+    assert (d["n_slots"] > 0) == (split_mma if flags else split)
+
+
+# whole prompts, whose partials cost more than the tail they save, and calls whose units fill the GPU, stay whole
+@pytest.mark.parametrize("heads,tokens,paths,queries", [(workloads.Heads(28, 4, 128), 1100, 1, 1100),
+                                                        (workloads.Heads(28, 4, 128), 2600, 1, 2600),
+                                                        (workloads.Heads(16, 2, 64), 1800, 1, 1800),
+                                                        (workloads.Heads(28, 4, 128), 2048, 32, 4),
+                                                        (workloads.Heads(28, 4, 128), 2048, 8, 64)])
+def test_blocks_left_whole(heads, tokens, paths, queries):
+    f = tp.Forest(heads.num_q_heads, heads.num_kv_heads, heads.head_dim, pool_blocks=paths * 82 + 8)
+    nodes = [f.add_root() for _ in range(paths)]
+    for x in nodes:
+        f.append(x, n_tokens=tokens)
+    assert tp.tp_debug_prefill_schedule(f.handle, nodes, [queries] * paths)["n_slots"] == 0
+    f.close()
 
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("flags", [0, tp.TP_MMA_SYNC])
 @pytest.mark.parametrize("heads", [workloads.Heads(28, 4, 128), workloads.Heads(16, 2, 64), workloads.Heads(12, 1, 128)])
-@pytest.mark.parametrize("tokens,queries", EDGES)
+@pytest.mark.parametrize("tokens,queries", [e[:2] for e in EDGES])
 def test_split_edges_against_the_oracle(tokens, queries, heads, flags):
     import torch
     if not torch.cuda.is_available():
