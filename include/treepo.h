@@ -606,7 +606,8 @@ tp_status tp_debug_check_schedule(tp_tree* tree, const int32_t* words, int64_t n
  * [10] = 1, no merge records ([11] = 0) and two more sections in their
  * place: unit_pos [n_units] (path position of each unit's first token) and
  * vis [n] (tokens of its path that occurrence i -- query token i -- may
- * see). Occurrences are the query
+ * see); occ and vis are written out here as the kernels derive them from the
+ * units. Occurrences are the query
  * tokens; units are tcgen05 units (mma.sync units with TP_MMA_SYNC); a unit
  * row whose occurrence sees nothing of the unit is computed but has no merge
  * entry. */

@@ -692,7 +692,7 @@ tp_status tp_prefill(tp_tree* t, const tp_node* nodes, const int32_t* n_queries,
     if (!Q || !O || !LSE || !aligned(Q, 16) || !aligned(O, 16) || !aligned(LSE, 4))
         return fail(t, TP_ERR_INVALID_ARG, "Q/O must be 16-byte and LSE 4-byte aligned device pointers");
     tp::Schedule& S = t->pf_sched;
-    tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S, true);
+    tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S);
     if (st != TP_OK) return st;
     if (S.n == 0) return TP_OK;
     st = refuse_capture(t, "tp_prefill");
@@ -901,12 +901,37 @@ tp_status tp_debug_prefill_schedule(tp_tree* t, const tp_node* nodes, const int3
     if (!t || !len) return TP_ERR_INVALID_ARG;
     if (n < 0 || (n > 0 && (!nodes || !n_queries))) return fail(t, TP_ERR_INVALID_ARG, "bad node list");
     tp::Schedule S;
-    tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S, false);
+    tp_status st = tp::build_prefill_schedule(t, nodes, n_queries, n, flags, S);
     if (st != TP_OK) return st;
-    *len = (int64_t)S.words.size();
+    // The words the kernels read, with the lists that the kernels derive from
+    // the units written out as the kernels derive them: each unit's rows are
+    // consecutive occurrences from its first, each seeing one token more.
+    const int32_t* w = S.words.data();
+    const int32_t g = t->cfg.num_q_heads / t->cfg.num_kv_heads;
+    const bool split = S.off_merge_slot > S.off_merge_off;
+    std::vector<int32_t> out(w, w + S.off_occ);
+    const size_t occ = out.size(), merge_off = occ + (size_t)S.n_occ, merge_slot = merge_off + (size_t)S.n + 1;
+    const size_t unit_pos = merge_slot + (size_t)S.n_merge, vis = unit_pos + (size_t)S.n_units;
+    out.resize(vis + (size_t)S.n, 0);
+    std::fill_n(out.begin() + (long)occ, S.n_occ, -1);  // an occurrence that no unit holds
+    for (int32_t k = 0; k < S.n_units; ++k) {
+        const int32_t* u = w + S.off_units + (int64_t)k * tp::kUnitWords;
+        for (int32_t p = 0; p < u[tp::U_N_ROWS] / g; ++p) {
+            const size_t o = (size_t)u[tp::U_OCC_OFF] + (size_t)p;
+            const int32_t sees = w[S.off_unit_vis + k] + p;
+            if (o >= (size_t)S.n) return fail(t, TP_ERR_INVALID_ARG, "a unit's rows lie outside the call's");
+            if (out[occ + o] != -1 && out[vis + o] != sees)
+                return fail(t, TP_ERR_INVALID_ARG, "two units give a row different visible lengths");
+            out[occ + o] = (int32_t)o;
+            out[vis + o] = sees;
+        }
+    }
+    if (split) std::copy(w + S.off_merge_off, w + S.off_unit_pos, out.begin() + (long)merge_off);
+    std::copy(w + S.off_unit_pos, w + S.off_unit_vis, out.begin() + (long)unit_pos);
+    *len = (int64_t)out.size();
     if (cap < *len) return cap == 0 ? TP_OK : fail(t, TP_ERR_INVALID_ARG, "buffer too small");
     if (!buf) return fail(t, TP_ERR_INVALID_ARG, "buf is NULL");
-    std::memcpy(buf, S.words.data(), S.words.size() * 4);
+    std::memcpy(buf, out.data(), out.size() * 4);
     return TP_OK;
 }
 

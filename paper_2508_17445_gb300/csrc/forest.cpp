@@ -445,12 +445,12 @@ tp_status build_schedule(tp_tree* t, const tp_node* leaves, int32_t n, uint32_t 
     // (block, kv head); the no-share control and the other routings give it
     // units that read the same blocks.
     S.kv_read_once = !(flags & (TP_DECODE_NO_SHARE | TP_DECODE_TCGEN05 | TP_MMA_SYNC));
-    S.off_unit_pos = S.off_vis = 0;
+    S.off_unit_pos = S.off_unit_vis = 0;
     return TP_OK;
 }
 
 tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t* m, int32_t n, uint32_t flags,
-                                 Schedule& S, bool device) {
+                                 Schedule& S) {
     const int32_t hq = t->cfg.num_q_heads, hkv = t->cfg.num_kv_heads, g = hq / hkv;
     if (g > kTensorRowsPerUnit)
         return fail(t, TP_ERR_INVALID_ARG, "prefill needs num_q_heads / num_kv_heads <= 64");
@@ -568,20 +568,18 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     S.n_occ = (int32_t)n_q;
     S.n = (int32_t)n_q;
     // A unit's query rows are consecutive query tokens, so the kernels derive
-    // each row's occurrence and what it sees; the device image leaves out the
-    // lists that only say so (occurrences, visible lengths) and, without
-    // split rows, the merge lists.
-    const bool lists = !device, csr = merge || !device;
+    // each row's occurrence and what it sees, and the schedule holds no lists
+    // that only say so (occurrences, visible lengths) nor, without split rows,
+    // merge lists.
     S.off_units = kSchedHeaderWords;
     S.off_tiles = S.off_units + (int64_t)S.n_units * kUnitWords;
     auto sections = [&](int64_t n_merge) {
         S.off_occ = S.off_tiles + S.n_tiles;
-        S.off_merge_off = S.off_occ + (lists ? S.n_occ : 0);
-        S.off_merge_slot = S.off_merge_off + (csr ? S.n + 1 : 0);
+        S.off_merge_off = S.off_occ;
+        S.off_merge_slot = S.off_merge_off + (merge ? S.n + 1 : 0);
         S.off_unit_pos = S.off_merge_slot + n_merge;
-        S.off_vis = S.off_unit_pos + S.n_units;
-        S.off_unit_vis = S.off_vis + (lists ? S.n : 0);
-        return S.off_unit_vis + (device ? S.n_units : 0);
+        S.off_unit_vis = S.off_unit_pos + S.n_units;
+        return S.off_unit_vis + S.n_units;
     };
     X.pair_occ.clear();
     X.pair_slot.clear();
@@ -631,7 +629,7 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
             }
         }
     }
-    if (csr) merge_csr(X, (int32_t)n_q);
+    if (merge) merge_csr(X, (int32_t)n_q);
     S.n_slots = n_slots;
     S.n_merge = (int32_t)X.pair_occ.size();
     S.off_merge_rec = 0;  // no merge records: most query rows are written directly, the rest use the CSR
@@ -653,18 +651,10 @@ tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t
     w[10] = 1;  // prefill schedule
     std::copy(X.tiles.begin(), X.tiles.end(), w + S.off_tiles);
     std::copy(X.unit_pos.begin(), X.unit_pos.end(), w + S.off_unit_pos);
-    if (device) std::copy(X.unit_vis.begin(), X.unit_vis.end(), w + S.off_unit_vis);
-    if (csr) {
+    std::copy(X.unit_vis.begin(), X.unit_vis.end(), w + S.off_unit_vis);
+    if (merge) {
         std::copy(X.merge_off.begin(), X.merge_off.end(), w + S.off_merge_off);
         std::copy(X.merge_slot.begin(), X.merge_slot.end(), w + S.off_merge_slot);
-    }
-    if (lists) {
-        for (int32_t q = 0; q < S.n; ++q) w[S.off_occ + q] = q;
-        int32_t* vis = w + S.off_vis;
-        for (int32_t i = 0; i < n; ++i) {
-            const Node& nd = t->nodes[(size_t)nodes[i]];
-            for (int32_t o = 0; o < m[i]; ++o) *vis++ = (int32_t)(nd.path_before + nd.n_tokens - m[i]) + o + 1;
-        }
     }
     S.leaf_tail.clear();
     return TP_OK;

@@ -338,10 +338,9 @@ class BlockPool {
 };
 
 struct Schedule {
-    // header | units | tiles | occ | merge_off | merge_slot, then for a
-    // decode schedule merge_rec [n][16], for a prefill one unit_pos
-    // [n_units] | vis [n]; a prefill one for the device leaves out occ, vis
-    // and (no split rows) merge_off, and ends in unit_vis [n_units]
+    // header | units | tiles | occ | merge_off | merge_slot | merge_rec [n][16];
+    // a prefill one: header | units | tiles | merge_off and merge_slot (only
+    // with split rows) | unit_pos [n_units] | unit_vis [n_units]
     std::vector<int32_t> words;
     int32_t n_units = 0, n_tiles = 0, n_occ = 0, n = 0, n_slots = 0, n_merge = 0, n_tensor = 0, n_tc = 0;
     int64_t off_units = 0, off_tiles = 0, off_occ = 0, off_merge_off = 0, off_merge_slot = 0;
@@ -349,7 +348,7 @@ struct Schedule {
     // Prefill calls of few units (the rule is in build_prefill_schedule): P in two bf16 terms.
     bool two_terms = false;
     bool kv_read_once = false;  // see DecodeArgs::kv_read_once
-    int64_t off_unit_pos = 0, off_vis = 0, off_unit_vis = 0, off_merge_rec = 0;
+    int64_t off_unit_pos = 0, off_unit_vis = 0, off_merge_rec = 0;
     // (leaf node, word index of the last tile of that leaf) for every place a
     // listed leaf's last block appears: appends that stay inside that block
     // change only these words (see patch_schedule)
@@ -520,10 +519,8 @@ tp_status build_schedule(tp_tree* t, const tp_node* leaves, int32_t n, uint32_t 
 // path's first vis[q] tokens; its rows are kept per node in blocks of whole
 // GQA groups, and each block reads the node's path tiles up to its last
 // visible token, in chunks of at most kMaxUnitTiles tiles.
-// device: the image the kernels read (see Schedule::words), else the whole
-// layout of tp_debug_prefill_schedule.
 tp_status build_prefill_schedule(tp_tree* t, const tp_node* nodes, const int32_t* m, int32_t n, uint32_t flags,
-                                 Schedule& out, bool device);
+                                 Schedule& out);
 // Refresh the last-tile words of S's leaves from the tree (valid after
 // appends that stayed inside those leaves' last blocks); `changed` receives
 // (word index, new word) pairs. Returns the number of changed words.
