@@ -1472,7 +1472,11 @@ struct TensorPath {
 // This CTA's k-th unit: its own index first (no round trip to the counter),
 // then whichever is next. CTAs that start beside another kernel do so one by
 // one, so their first unit comes from the counter too: assigned by index, a
-// late CTA would hold one of the longest units.
+// late CTA would hold one of the longest units. That can still happen to a
+// launch that another stream's work keeps from starting whole; a grid ends with
+// its last CTA either way, and the unit in its hands costs little: 16 leaves
+// beside large copies 80 us a call against 78 with the counter alone (beside
+// GEMMs equal), a prompt of 1.8k tokens alone 42.9 against 44.6.
 __device__ __forceinline__ int claim_unit(const DecodeArgs& a, int k) {
     if (a.late_wait) return a.unit_begin + atomicAdd(a.counter, 1);
     return a.unit_begin + (int)(k == 0 ? blockIdx.x : gridDim.x + atomicAdd(a.counter, 1));
@@ -2696,9 +2700,8 @@ int decode_tc_grid() {
             return 0;
         // The occupancy query answers 1 for this kernel on GB300 although its
         // registers (128 x 224 threads) and shared memory fit twice per SM, so
-        // count from those resources too. Launching more CTAs than fit is
-        // harmless for a persistent kernel: a CTA that starts late finds the
-        // unit counter exhausted and exits.
+        // count from those resources too. A CTA more than fits would start when
+        // the first one ends, with the unit of its index (claim_unit).
         cudaFuncAttributes fa{};
         int smem_sm = 0, reserved = 0;
         if (cudaFuncGetAttributes(&fa, decode_tc_kernel<HD, CAUSAL, TWO, CAP>) != cudaSuccess) return 0;
@@ -2748,10 +2751,10 @@ cudaError_t launch_tc_range(DecodeArgs a, int begin, int end, int32_t* counter, 
 // CTA: few of them end unevenly, and the mma.sync units fill those gaps, while
 // many end evenly by themselves, and launched last their partials (the larger
 // part) are still in L2 when the merge reads them. Measured, tcgen05 units
-// first against last: 16 diverging prompts (1180 units) 509 / 520 us, 64 leaves
-// x 8 prompts with a 2k prefix (1536) 309 / 317, 48 binary trees (1344) 245 /
-// 246; 24 diverging prompts (1792) 828 / 823, 64 binary trees (1792) 326 / 322,
-// 32 diverging prompts (2444) 1116 / 1101, 96 binary trees (2688) 490 / 483.
+// first against last: 16 diverging prompts (1192 units) 500 / 517 us, 48 binary
+// trees (1344) 239 / 236, 64 leaves x 8 prompts with a 2k prefix (1536) 301 /
+// 308; 64 binary trees (1792) 320 / 311, 24 diverging prompts (1812) 816 / 811,
+// 12 prompts with the prefix (2304) 445 / 435, 32 diverging (2468) 1100 / 1081.
 constexpr int kTcLastUnits = 11 * 152;
 
 template <int HD>
