@@ -134,7 +134,8 @@ void append_tokens_commit(tp_tree* t, const tp_node* nodes, int32_t n, int64_t n
 
 int32_t step_patch(tp_tree* t, const tp_node* nodes, int32_t n, bool stays, uint64_t before, bool* patched) {
     *patched = stays && t->sched_valid && t->sched_version == before && t->sched_struct == t->struct_version &&
-               t->sched_stream == t->stream && t->sched_leaves.size() == (size_t)n && std::equal(nodes, nodes + n, t->sched_leaves.begin());
+               t->sched_stream == t->stream && t->sched_leaves.size() == (size_t)n &&
+               std::equal(nodes, nodes + n, t->sched_leaves.begin());
     return *patched ? patch_schedule(t, t->sched, t->patch_words) : 0;
 }
 
