@@ -2455,8 +2455,8 @@ __device__ __forceinline__ void merge_batch(const MergeArgs& a, int qh, int lane
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const bool on = j0 + u < cnt;
-        const int64_t sl = __shfl_sync(0xffffffffu, slot, on ? j0 + u : j0);  // off: re-read row j0, weight 0
-        wj[u] = __shfl_sync(0xffffffffu, w, on ? j0 + u : j0) * (on ? 1.f : 0.f);
+        const int64_t sl = __shfl_sync(0xffffffffu, slot, on ? j0 + u : j0);  // off: re-read row j0, not added
+        wj[u] = __shfl_sync(0xffffffffu, w, on ? j0 + u : j0);
         const float* src = a.part_o + (sl * a.hq + qh) * HD + lane * DPL;
         srcs[u] = on ? src : nullptr;
         if constexpr (DPL == 4) {
@@ -2469,8 +2469,9 @@ __device__ __forceinline__ void merge_batch(const MergeArgs& a, int qh, int lane
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u)
+        if (j0 + u < cnt)  // (a weight of 0 would make NaN of an infinite partial)
 #pragma unroll
-        for (int d = 0; d < DPL; ++d) acc[d] += wj[u] * x[u][d];
+            for (int d = 0; d < DPL; ++d) acc[d] += wj[u] * x[u][d];
     __syncwarp();
     if ((lane & (kLanesPerLine - 1)) == 0)
 #pragma unroll
@@ -2514,9 +2515,9 @@ __device__ __forceinline__ void merge_chunk(const MergeArgs& a, int qh, int lane
     for (int d = 0; d < DPL; ++d) acc[d] *= keep;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const float wu = __shfl_sync(0xffffffffu, w, u) * (u < cnt ? 1.f : 0.f);
+        const float wu = __shfl_sync(0xffffffffu, w, u);
 #pragma unroll
-        for (int d = 0; d < DPL; ++d) acc[d] += wu * x0[u][d];
+        for (int d = 0; d < DPL; ++d) acc[d] += wu * (u < cnt ? x0[u][d] : 0.f);
     }
     constexpr int kLanesPerLine = 128 / (DPL * 4);
     __syncwarp();
