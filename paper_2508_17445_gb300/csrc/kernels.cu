@@ -211,12 +211,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// Second terms of two probabilities: what their bf16 roundings (a pair, as
-// packed) leave out, in bf16 again.
-__device__ __forceinline__ uint32_t second_terms(float p0, float p1, uint32_t first) {
-    return pack_bf16(p0 - __uint_as_float(first << 16), p1 - __uint_as_float(first & 0xffff0000u));
-}
-
 // 32-byte global store (sm_100 and later); dst must be 32-byte aligned
 __device__ __forceinline__ void st_global_v8(void* dst, const uint32_t* w) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]),
@@ -257,6 +251,22 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
     uint64_t r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
+}
+
+// Two probabilities in two bf16 terms each (pairs as packed): the first is the
+// probability's upper half, the second what that leaves out (less than 2^-7 of
+// it), plus 2^-23 of the probability so that both terms are above 0 wherever it
+// is: an infinite V stays infinite in O instead of 0 or a negative times it
+// making NaN.
+__device__ __forceinline__ void bf16_terms(float p0, float p1, uint32_t& first, uint32_t& second) {
+    const uint32_t u0 = __float_as_uint(p0), u1 = __float_as_uint(p1);
+    first = __byte_perm(u0, u1, 0x7632);
+    const uint64_t minus = f2_pack(__uint_as_float((u0 & 0xffff0000u) | 0x80000000u),
+                                   __uint_as_float((u1 & 0xffff0000u) | 0x80000000u));
+    constexpr float kUp = 1.f + 1.f / (1 << 23);
+    float r0, r1;
+    f2_unpack(f2_fma(f2_pack(p0, p1), f2_pack(kUp, kUp), minus), r0, r1);
+    second = pack_bf16(r0, r1);
 }
 
 // bf16 pair in a 32-bit word -> two fp32 (exact: bf16 is the top half of fp32)
@@ -1361,11 +1371,12 @@ struct TensorPath {
                         const float p2 = fast_exp2(s[j][2] - m_use[1]), p3 = fast_exp2(s[j][3] - m_use[1]);
                         l_run[0] += p0 + p1;
                         l_run[1] += p2 + p3;
-                        pa[2 * j] = pack_bf16(p0, p1);
-                        pa[2 * j + 1] = pack_bf16(p2, p3);
-                        if constexpr (CAUSAL) {
-                            pb[2 * j] = second_terms(p0, p1, pa[2 * j]);
-                            pb[2 * j + 1] = second_terms(p2, p3, pa[2 * j + 1]);
+                        if (CAUSAL && a.two_terms) {
+                            bf16_terms(p0, p1, pa[2 * j], pb[2 * j]);
+                            bf16_terms(p2, p3, pa[2 * j + 1], pb[2 * j + 1]);
+                        } else {
+                            pa[2 * j] = pack_bf16(p0, p1);
+                            pa[2 * j + 1] = pack_bf16(p2, p3);
                         }
                     }
 #pragma unroll
@@ -2288,8 +2299,10 @@ __device__ void tc_consume(const DecodeArgs& a, CtlTc& c) {
                                   x0, x1);
                         const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
                         acc[(t >> 1) & 1] = f2_add(acc[(t >> 1) & 1], f2_pack(p0, p1));
-                        pw[h * 16 + t / 2] = pack_bf16(p0, p1);
-                        if constexpr (TWO) pl[h * 16 + t / 2] = second_terms(p0, p1, pw[h * 16 + t / 2]);
+                        if constexpr (TWO)
+                            bf16_terms(p0, p1, pw[h * 16 + t / 2], pl[h * 16 + t / 2]);
+                        else
+                            pw[h * 16 + t / 2] = pack_bf16(p0, p1);
                     }
                 float s0, s1, s2, s3;
                 f2_unpack(acc[0], s0, s1);

@@ -125,7 +125,7 @@ def test_masked_last_stages(tokens, heads):
 
 
 # Calls of few units hold each probability in two bf16 terms, split rows or not: what they leave out is 2^-16 of the
-# probability, so O is off by its own rounding (half a unit in the last of its 8 places) and, with what fp32 sums and exp2
+# probability (2^-8 of a second term below 2^-7 of it, halved by rounding), so O is off by its own rounding (half a unit in the last of its 8 places) and, with what fp32 sums and exp2
 # add to the scores and the sums, 2^-15 of A = sum p |v|. (One bf16 term leaves out up to 2^-8 of each probability, in sum
 # ~2^-13 A over some hundred tokens.)
 # Schedules of both parameter sizes, uploaded, and with split rows
@@ -152,4 +152,30 @@ def test_probabilities_in_two_terms(tokens, queries, heads, flags):
     d_o = np.abs(O[rows].float().cpu().numpy().astype(np.float64) - o_ref)
     assert (d_o <= 2.0 ** (np.floor(np.log2(np.abs(o_ref))) - 8) + 2.0 ** -15 * a_ref).all()
     assert np.abs(LSE[rows].cpu().numpy().astype(np.float64) - lse_ref).max() <= 5e-5
+    f.close()
+
+
+# Infinite values come through as in calls with one term: both terms of a probability are above 0 where it is (rows that do
+# not see the value are left out: a masked probability of 0 times infinity is NaN there, as in every tensor-core product;
+# whole tiles, since what a short one leaves of its slot is multiplied by 0 too)
+@pytest.mark.gpu
+@pytest.mark.parametrize("flags", [0, tp.TP_MMA_SYNC])
+@pytest.mark.parametrize("tokens,queries", [(128, 128), (704, 704), (2112, 40)])
+def test_infinite_values(tokens, queries, flags):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    g = torch.Generator(device="cuda:0").manual_seed(tokens)
+    K, V = (torch.randn((tokens, 2, 128), generator=g, device="cuda:0").to(torch.bfloat16) for _ in range(2))
+    V[10, 0, 5], V[20, 1, 7] = float("inf"), float("-inf")
+    Q = torch.randn((queries, 8, 128), generator=g, device="cuda:0").to(torch.bfloat16)
+    f = tp.Forest(8, 2, 128, pool_blocks=128, device="cuda:0")
+    r = f.add_root()
+    f.append(r, K, V)
+    O, _ = f.prefill([r], [queries], Q, flags)
+    f.sync()
+    see = O[-min(queries, tokens - 20):]
+    assert (see[:, :4, 5] == float("inf")).all() and (see[:, 4:, 7] == float("-inf")).all()
+    see[:, :4, 5], see[:, 4:, 7] = 0, 0
+    assert torch.isfinite(see.float()).all()
     f.close()
